@@ -21,7 +21,7 @@ import paper_1211_4575_gb300 as pp
 
 DEVICE = "cuda"
 # Past this many particle-steps the FP64 integration takes longer than about 20 s.
-EXACT_PARTICLE_STEPS = 7.0e8
+EXACT_PARTICLE_STEPS = 4.1e8
 
 # Values a case that does not state them takes.
 DEFAULTS = dict(kind="thermal", shape=3, precision="mixed", pusher="vay", steps=10, walls="", solver="implicit",
@@ -53,11 +53,11 @@ def listed():
         # The numerical-heating run at a size that nearly fills the GPU, with its energy series.
         dict(name="thermal_64_energies", kind="thermal", nx=64, ny=64, nz=64, ppc=32, steps=10, output="energies"),
         # The numerical-heating run at full size.
-        dict(name="thermal_128", kind="thermal", nx=128, ny=128, nz=128, ppc=32, steps=5),
+        dict(name="thermal_128", kind="thermal", nx=128, ny=128, nz=128, ppc=32, steps=3),
         # The Gamma = 10 beam through an electron-ion background: the production run and the largest.
         dict(name="beam_256", kind="beam", nx=256, ny=128, nz=128, ppc=16, steps=10),
         # The largest served request, few particles per cell: the mesh weighs most here.
-        dict(name="weibel_192", kind="weibel", nx=192, ny=192, nz=192, ppc=8, steps=5),
+        dict(name="weibel_192", kind="weibel", nx=192, ny=192, nz=192, ppc=8, steps=3),
         # A plasma between reflecting walls on x.
         dict(name="walls_64", kind="heating", nx=64, ny=64, nz=64, ppc=16, walls="x", steps=10),
         # The original method that the paper compares with: direct current, explicit fields, filtered E and B.
