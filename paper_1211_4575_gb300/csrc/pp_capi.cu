@@ -577,6 +577,12 @@ static bool cells_mode(const Ctx *c) {
     return !c->fp64 && (m == PP_DEPOSIT_CELLS || m == PP_DEPOSIT_AUTO) && cells_supported(*c);
 }
 
+// Either kernel that starts from particles sorted in this step: that one, or
+// on meshes its tiles do not divide the row kernel (automatic deposit).
+static bool sorted_mode(const Ctx *c) {
+    return cells_mode(c) || (c->d.deposit_mode == PP_DEPOSIT_AUTO && rows_supported(*c));
+}
+
 // The parts of a particle phase around its kernel launch: before it, the
 // per-step sort of the per-step sorted kernel when the particles moved, and
 // the cleared current; after it, the ghost fold, the images' current between
@@ -618,7 +624,7 @@ static int particle_post(Ctx *c, int only) {
 
 static int particle_phase(Ctx *c, int only) {
     NvtxRange nvtx("pp particle phase");
-    const bool cells = only < 0 && cells_mode(c);
+    const bool cells = only < 0 && sorted_mode(c);
     if (int r = particle_pre(c, cells)) return r;
     bool all_sorted = true;
     for (int s = 0; s < c->nspecies; ++s) all_sorted = all_sorted && (c->sp[s].sorted || c->sp[s].n == 0);
@@ -626,7 +632,8 @@ static int particle_phase(Ctx *c, int only) {
     bool tiled = !c->fp64 && !cells && (m == PP_DEPOSIT_TILED || m == PP_DEPOSIT_CELLS ||
                                         (m == PP_DEPOSIT_AUTO && tiled_supported(*c) && all_sorted));
     if (cells) {
-        CU(launch_particles_cells(*c));
+        if (cells_mode(c)) CU(launch_particles_cells(*c));
+        else CU(launch_particles_rows(*c));
         if (c->prof) ++c->prof_particle_launches;
     } else if (tiled && only < 0) {
         CU(launch_particles_tiled_all(*c));
@@ -808,8 +815,8 @@ static int step_body(Ctx *c, bool sort, bool filter) {
 static bool graph_matches(const Ctx *c, const StepGraph &G, bool sort, bool filter) {
     if (!G.valid || G.sort != sort || G.filter != filter || G.J0 != c->J[0]) return false;
     // freshness, a pending permutation and valid keys change what a step
-    // launches only for the per-step sorted kernel (elsewhere they stay false)
-    const bool cells = cells_mode(c);
+    // launches only for the per-step sorted kernels (elsewhere they stay false)
+    const bool cells = sorted_mode(c);
     for (int s = 0; s < c->nspecies; ++s) {
         if (G.buf[s] != c->sp[s].buf || G.sorted[s] != c->sp[s].sorted) return false;
         if (cells && (G.fresh[s] != c->sp[s].fresh || G.pending[s] != c->sp[s].perm_pending ||

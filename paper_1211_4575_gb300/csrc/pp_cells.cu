@@ -42,8 +42,7 @@
 // overflow, and after the chunk the nodes its cells reach are added into the
 // FP32 mesh (one global atomic per nonzero node).  A piece's sum is FP32 in
 // registers and is rounded to the unit once.
-#include "pp_internal.cuh"
-#include "pp_particle_common.cuh"
+#include "pp_sorted.cuh"
 #include "pp_tma.cuh"
 
 namespace pp {
@@ -171,53 +170,11 @@ struct CellsCurrentAcc {
     }
 };
 
-struct CellsSpecies {
-    MixedParticles p;            // read: slot i of the sorted order is p[perm[i]] (p[i] without perm)
-    MixedParticles out;          // written: the new state of slot i, in the sorted order
-    const int32_t *perm;         // pending sort permutation, or null
-    int32_t *keys;               // written: the sort key of each slot's new state
-    const int32_t *cell_start;   // per sort key, tile-major
-    float qmdt;
-    float kdt;                   // radiative cooling K / dt (0 = off)
-    float jscale[3];             // -q w dx_a / dt
-};
+using CellsSpecies = SortedSpecies;
 
-struct CellsArgs {
+struct CellsArgs : SortedArgs {
     CUtensorMap tmap[6];         // E_x, E_y, E_z, B_x, B_y, B_z: boxes of kWG^3 nodes
-    Geom g;
-    const float *E[3];
-    const float *B[3];
-    float *J[3];
-    float dtdx[3];
-    int nt[3];
-    int ns;
-    CellsSpecies sp[PP_MAX_SPECIES];
-    int *status;
-    int wall[3];                 // walls at 0 and wall[a] cells on axis a; 0 = periodic
-    double esc;                  // open end: outgoing particles below x = esc cells leave; 0 = off
-    int32_t dead_key;            // sort key of a particle that left: after every cell's keys
 };
-
-// Sort key of a particle in cell (x, y, z) with offsets o (the key of the cell
-// sort: its 8^3 tile in tile order, its cell in the tile, the octant of the
-// cell that holds it), or dead_key for a particle that left.
-__device__ __forceinline__ int32_t sort_key(const CellsArgs &T, int32_t cw, const float (&o)[3]) {
-    if (cw < 0) return T.dead_key;
-    int x, y, z;
-    unpack_cell(cw, x, y, z);
-    const int tile = ((z / kT) * T.nt[1] + y / kT) * T.nt[0] + x / kT;
-    const int cell = ((z % kT) * kT + y % kT) * kT + x % kT;
-    const int oct = (o[0] >= 0.5f ? 1 : 0) | (o[1] >= 0.5f ? 2 : 0) | (o[2] >= 0.5f ? 4 : 0);
-    return (tile * kTCells + cell) * kSubKeys + oct;
-}
-
-__device__ __forceinline__ void store(const CellsArgs &T, const CellsSpecies &S, int64_t i, int32_t cw,
-                                      const float (&o)[3], const float (&u)[3]) {
-    S.out.cell[i] = cw;
-    S.out.ox[i] = o[0]; S.out.oy[i] = o[1]; S.out.oz[i] = o[2];
-    S.out.ux[i] = u[0]; S.out.uy[i] = u[1]; S.out.uz[i] = u[2];
-    S.keys[i] = sort_key(T, cw, o);
-}
 
 // Deposit group of a particle: its cell in the tile, and for even orders the
 // octant of the cell it sits in (the support start on integer nodes is
@@ -628,7 +585,7 @@ __device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int tile, f
                     // not in its sorted tile: cannot happen after a sort; left unmoved and flagged
                     atomicOr(T.status, ST_RANGE);
                     s_grp[q] = kSkip;
-                    store(T, S, idx, cw0, xi0, u);
+                    store_sorted(T, S, idx, cw0, xi0, u);
                     continue;
                 }
                 const float u0[3] = {u[0], u[1], u[2]};
@@ -657,7 +614,7 @@ __device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int tile, f
                 if (!ok) {   // leave the particle unchanged and flag the step
                     atomicOr(T.status, isfinite(u[0] + u[1] + u[2]) ? ST_CFL : ST_NAN);
                     s_grp[q] = (uint16_t)(grp | kSkip);
-                    store(T, S, idx, cw0, xi0, u0);
+                    store_sorted(T, S, idx, cw0, xi0, u0);
                     continue;
                 }
 #pragma unroll
@@ -689,7 +646,7 @@ __device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int tile, f
                 } else {
                     cwd = pack_cell(ncx, ncy, ncz);
                 }
-                store(T, S, idx, cwd, xi1, u);
+                store_sorted(T, S, idx, cwd, xi1, u);
             }
 #if PP_CELLS_FIXED
             if (threadIdx.x < 3) {   // previous chunk's values were last read before the barrier above
@@ -948,63 +905,14 @@ bool cells_supported(const Ctx &c) {
 // arrays; any = false when no species holds particles.
 static cudaError_t cells_args(const Ctx &c, CellsArgs &T, bool &any) {
     any = false;
-    T.g = c.g;
-    const double h[3] = {c.d.dx, c.d.dy, c.d.dz};
-    for (int d = 0; d < 3; ++d) {
-        T.E[d] = (const float *)c.E[d];
-        T.B[d] = (const float *)c.B[d];
-        T.J[d] = (float *)c.J[d];
-        T.dtdx[d] = (float)(c.drift_dt / h[d]);
-        T.nt[d] = c.ntile[d];
-    }
+    sorted_args(c, T);
     const int box[3] = {kWG, kWG, kWG};
     for (int comp = 0; comp < 6; ++comp) {
         cudaError_t e = encode_box_map(&T.tmap[comp], comp < 3 ? T.E[comp] : T.B[comp - 3], c.g.P, box);
         if (e != cudaSuccess) return e;
     }
-    T.ns = 0;
-    for (int s = 0; s < c.nspecies; ++s) {
-        const Species &S = c.sp[s];
-        if (S.n == 0) continue;
-        CellsSpecies &t = T.sp[T.ns++];
-        t.p = MixedParticles{S.cell, S.ox, S.oy, S.oz, S.fux, S.fuy, S.fuz};
-        int32_t *c2 = (int32_t *)S.alt;
-        float *f2 = (float *)(c2 + S.cap);
-        t.out = MixedParticles{c2, f2, f2 + S.cap, f2 + 2 * S.cap, f2 + 3 * S.cap, f2 + 4 * S.cap, f2 + 5 * S.cap};
-        t.perm = S.perm_pending ? S.perm : nullptr;
-        t.keys = S.keys;
-        t.cell_start = S.cell_start;
-        t.qmdt = (float)(S.q * c.kick_dt / S.m);
-        t.kdt = (float)(c.kick_dt != 0.0 ? S.rad / c.kick_dt : 0.0);
-        for (int d = 0; d < 3; ++d) t.jscale[d] = (float)(-S.q * S.w * h[d] / c.drift_dt);
-    }
-    T.status = c.d_status;
-    for (int d = 0; d < 3; ++d) T.wall[d] = c.wall[d];
-    T.esc = c.escape_now;
-    T.dead_key = (int32_t)c.nkeys;
     any = T.ns > 0;
     return cudaSuccess;
-}
-
-static bool cells_ready(const Ctx &c) {
-    for (int s = 0; s < c.nspecies; ++s)
-        if (c.sp[s].n > 0 && !c.sp[s].fresh) return false;
-    return true;
-}
-
-// After the launch: every slot of the sorted order holds its particle's new
-// state in the other buffer, with its next sort key.
-static void cells_after(Ctx &c) {
-    for (int s = 0; s < c.nspecies; ++s) {
-        Species &S = c.sp[s];
-        if (S.n == 0) continue;
-        void *old = S.buf;
-        S.buf = S.alt;
-        S.alt = old;
-        S.bind(false);
-        S.perm_pending = false;
-        S.keys_valid = true;
-    }
 }
 
 template <class K>
@@ -1016,7 +924,7 @@ static cudaError_t smem_attr(K kernel, unsigned long long &done) {
 // sorted since its particles last moved (Species::fresh).
 cudaError_t launch_particles_cells(Ctx &c) {
     if (!cells_supported(c)) return cudaErrorInvalidConfiguration;
-    if (!cells_ready(c)) return cudaErrorInvalidValue;
+    if (!sorted_ready(c)) return cudaErrorInvalidValue;
     CellsArgs T;
     bool any = false;
     cudaError_t ea = cells_args(c, T, any);
@@ -1045,7 +953,7 @@ cudaError_t launch_particles_cells(Ctx &c) {
     ++c.nlaunch;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    cells_after(c);
+    sorted_after(c);
     return cudaSuccess;
 }
 
@@ -1066,7 +974,7 @@ cudaError_t launch_particles_cells_batch(Ctx *const *ctxs, int n, cudaStream_t s
     int order[4096], m = 0;
     for (int k = 0; k < n && m < 4096; ++k) {
         Ctx &c = *ctxs[k];
-        if (!cells_supported(c) || !cells_ready(c)) return cudaErrorInvalidValue;
+        if (!cells_supported(c) || !sorted_ready(c)) return cudaErrorInvalidValue;
         bool any = false;
         cudaError_t ea = cells_args(c, A[m], any);
         if (ea != cudaSuccess) return ea;
@@ -1122,7 +1030,7 @@ cudaError_t launch_particles_cells_batch(Ctx *const *ctxs, int n, cudaStream_t s
     for (int a = 0; a < m; ++a) {
         Ctx &c = *ctxs[order[a]];
         ++c.nlaunch;
-        cells_after(c);
+        sorted_after(c);
     }
     return cudaSuccess;
 }

@@ -95,13 +95,36 @@ __device__ __forceinline__ int support(R xi, bool half, R (&w)[O + 1]) {
     return (int)fl;
 }
 
+// 1 / sqrt(x), x >= 1.  FP32: one Newton-Raphson step on the hardware estimate
+// (y += y/2 (1 - x y^2), error below one ulp), a quarter of the instructions of
+// a correctly rounded square root and division; infinity gives 0.
+__device__ __forceinline__ double inv_sqrt(double x) { return 1.0 / sqrt(x); }
+__device__ __forceinline__ float inv_sqrt(float x) {
+    const float y = rsqrtf(x);
+    const float r = fmaf(0.5f * y, fmaf(-(x * y), y, 1.0f), y);
+    return x < 3.0e38f ? r : y;
+}
+
+// sqrt(x) of x > 0 and 1 / x of x >= 1, likewise.
+__device__ __forceinline__ double fast_sqrt(double x) { return sqrt(x); }
+__device__ __forceinline__ float fast_sqrt(float x) {
+    const float y = rsqrtf(x), s = x * y;
+    const float r = fmaf(0.5f * y, fmaf(-s, s, x), s);
+    return x < 3.0e38f ? r : x;
+}
+__device__ __forceinline__ double inv(double x) { return 1.0 / x; }
+__device__ __forceinline__ float inv(float x) {
+    const float y = __fdividef(1.0f, x);
+    return x < 1.0e38f ? fmaf(y, fmaf(-x, y, 1.0f), y) : y;
+}
+
 // ---------------------------------------------------------------------------
 // Relativistic pushers (Sec. III "Particle motion"), c = 1.
 // qmdt = q dt / m.  u: proper velocity at t - dt/2 in, t + dt/2 out.
 // ---------------------------------------------------------------------------
 template <typename R>
 __device__ __forceinline__ void push_vay(R qmdt, const R (&E)[3], const R (&B)[3], R (&u)[3]) {
-    R ginv = R(1) / sqrt(R(1) + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+    R ginv = inv_sqrt(R(1) + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
     R h = R(0.5) * qmdt;
     R tx = h * B[0], ty = h * B[1], tz = h * B[2];
     // u' = u + qdt/m E + v x tau
@@ -112,10 +135,9 @@ __device__ __forceinline__ void push_vay(R qmdt, const R (&E)[3], const R (&B)[3
     R tau2 = tx * tx + ty * ty + tz * tz;
     R us = px * tx + py * ty + pz * tz;
     R sigma = R(1) + px * px + py * py + pz * pz - tau2;
-    R gnew = sqrt(R(0.5) * (sigma + sqrt(sigma * sigma + R(4) * (tau2 + us * us))));
-    R gi = R(1) / gnew;
+    R gi = inv_sqrt(R(0.5) * (sigma + fast_sqrt(sigma * sigma + R(4) * (tau2 + us * us))));
     tx *= gi; ty *= gi; tz *= gi;
-    R s = R(1) / (R(1) + tx * tx + ty * ty + tz * tz);
+    R s = inv(R(1) + tx * tx + ty * ty + tz * tz);
     R pt = px * tx + py * ty + pz * tz;
     u[0] = s * (px + pt * tx + (py * tz - pz * ty));
     u[1] = s * (py + pt * ty + (pz * tx - px * tz));
@@ -126,12 +148,12 @@ template <typename R>
 __device__ __forceinline__ void push_boris(R qmdt, const R (&E)[3], const R (&B)[3], R (&u)[3]) {
     R h = R(0.5) * qmdt;
     R mx = u[0] + h * E[0], my = u[1] + h * E[1], mz = u[2] + h * E[2];
-    R gi = R(1) / sqrt(R(1) + mx * mx + my * my + mz * mz);
+    R gi = inv_sqrt(R(1) + mx * mx + my * my + mz * mz);
     R tx = h * B[0] * gi, ty = h * B[1] * gi, tz = h * B[2] * gi;
     R ax = mx + (my * tz - mz * ty);
     R ay = my + (mz * tx - mx * tz);
     R az = mz + (mx * ty - my * tx);
-    R f = R(2) / (R(1) + tx * tx + ty * ty + tz * tz);
+    R f = R(2) * inv(R(1) + tx * tx + ty * ty + tz * tz);
     R sx = f * tx, sy = f * ty, sz = f * tz;
     u[0] = mx + (ay * sz - az * sy) + h * E[0];
     u[1] = my + (az * sx - ax * sz) + h * E[1];
@@ -164,15 +186,10 @@ __device__ __forceinline__ void radiate(R kdt, const R (&um)[3], R (&u)[3]) {
 // when the species radiates (kdt != 0, uniform over a launch).
 template <int PUSH, typename R>
 __device__ __forceinline__ void push_particle(R qmdt, R kdt, const R (&E)[3], const R (&B)[3], R (&u)[3]) {
-    if (kdt != R(0)) {
-        R um[3] = {u[0], u[1], u[2]};
-        if (PUSH == PP_BORIS) push_boris<R>(qmdt, E, B, u);
-        else push_vay<R>(qmdt, E, B, u);
-        radiate<R>(kdt, um, u);
-    } else {
-        if (PUSH == PP_BORIS) push_boris<R>(qmdt, E, B, u);
-        else push_vay<R>(qmdt, E, B, u);
-    }
+    R um[3] = {u[0], u[1], u[2]};
+    if (PUSH == PP_BORIS) push_boris<R>(qmdt, E, B, u);
+    else push_vay<R>(qmdt, E, B, u);
+    if (kdt != R(0)) radiate<R>(kdt, um, u);
 }
 
 // ---------------------------------------------------------------------------
@@ -633,6 +650,8 @@ cudaError_t launch_particles_tiled_all(Ctx &c);
 bool tiled_supported(const Ctx &c);
 cudaError_t launch_particles_cells(Ctx &c);
 bool cells_supported(const Ctx &c);
+cudaError_t launch_particles_rows(Ctx &c);
+bool rows_supported(const Ctx &c);
 // batched form: one launch over the tiles of many contexts (same shape order,
 // pusher and boundary kind); scratch = device memory the caller owns
 struct CellsBatchScratch {
