@@ -130,30 +130,30 @@ static int setup_operators(Ctx *c) {
         c->lap[s] = -acc;    // l_s = sum_p t_p t_{s-p} = -sum_p t_{p+s} t_p by antisymmetry
     }
     // high-order current taps
-    std::vector<double> host(3 * kMaxTaps, 0.0);
-    double eps = c->fp64 ? 1e-18 : 1e-10;
+    double *host = c->h_taps;
     for (int a = 0; a < 3; ++a) {
         c->ntaps[a] = 0;
         if (c->d.field_order == 2) continue;
         int n = c->g.n[a];
         std::vector<double> gi;
         circulant_inverse(n, c->fd, gi);
-        if (n <= kMaxTaps) {
+        // The taps decay geometrically.  FP32: those above 1e-10 of the first
+        // (8 to each side at 6th order); FP64: twice that reach, 1e-20.  A mesh
+        // no longer than that takes the whole period.
+        int K = 1;
+        while (K < n / 2 && fabs(gi[K + 1]) > 1e-10 * fabs(gi[0])) ++K;
+        if (c->fp64) K *= 2;
+        if (K > (kMaxTaps - 1) / 2) K = (kMaxTaps - 1) / 2;
+        if (2 * K + 1 >= n && n <= kMaxTaps) {
             c->full_circ[a] = true;
             c->ntaps[a] = n;
             for (int m = 0; m < n; ++m) host[a * kMaxTaps + m] = gi[m];
         } else {
-            int K = 1;
-            while (K < n / 2 && K < (kMaxTaps - 1) / 2 && fabs(gi[K + 1]) > eps * fabs(gi[0])) ++K;
             c->full_circ[a] = false;
             c->ntaps[a] = 2 * K + 1;
             for (int m = 0; m <= 2 * K; ++m) host[a * kMaxTaps + m] = gi[abs(m - K)];
         }
     }
-    cudaError_t e = cudaMalloc(&c->taps, sizeof(double) * 3 * kMaxTaps);
-    if (e != cudaSuccess) return fail(c, PP_ECUDA, "taps: %s", cudaGetErrorString(e));
-    e = cudaMemcpy(c->taps, host.data(), sizeof(double) * 3 * kMaxTaps, cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return fail(c, PP_ECUDA, "taps copy: %s", cudaGetErrorString(e));
     // Chebyshev bounds of A = 1 - alpha^2 dt^2 L for every solve step the
     // context takes: the step dt and the drifts of the 4th-order substeps
     double a[4], b[4];
@@ -311,7 +311,6 @@ extern "C" int pp_destroy(pp_ctx *p) {
     cudaFree(c->mesh);
     cudaFree(c->rho);
     cudaFree(c->G0);
-    cudaFree(c->taps);
     cudaFree(c->counts);
     cudaFree(c->scan_tmp);
     cudaFree(c->d_status);
@@ -600,7 +599,8 @@ static int particle_pre(Ctx *c, bool cells) {
         }
     }
     CU(launch_zero_J(*c));
-    CU(cudaMemsetAsync(c->d_nslow, 0, sizeof(unsigned long long), c->st));
+    if (c->nslow_set) CU(cudaMemsetAsync(c->d_nslow, 0, sizeof(unsigned long long), c->st));
+    c->nslow_set = false;
     CU(prof_mark(c, PH_PARTICLE, true));
     return PP_OK;
 }
@@ -636,6 +636,7 @@ static int particle_phase(Ctx *c, int only) {
         else CU(launch_particles_rows(*c));
         if (c->prof) ++c->prof_particle_launches;
     } else if (tiled && only < 0) {
+        c->nslow_set = true;   // the only kernel that counts
         CU(launch_particles_tiled_all(*c));
         if (c->prof) ++c->prof_particle_launches;
     } else {
@@ -813,7 +814,7 @@ static int step_body(Ctx *c, bool sort, bool filter) {
 }
 
 static bool graph_matches(const Ctx *c, const StepGraph &G, bool sort, bool filter) {
-    if (!G.valid || G.sort != sort || G.filter != filter || G.J0 != c->J[0]) return false;
+    if (!G.valid || G.sort != sort || G.filter != filter || G.J0 != c->J[0] || G.B0 != c->B[0]) return false;
     // freshness, a pending permutation and valid keys change what a step
     // launches only for the per-step sorted kernels (elsewhere they stay false)
     const bool cells = sorted_mode(c);
@@ -832,6 +833,9 @@ static void graph_save_after(const Ctx *c, StepGraph &G) {
     for (int a = 0; a < 3; ++a) {
         G.J_after[a] = c->J[a];
         G.Jt_after[a] = c->Jt[a];
+        G.B_after[a] = c->B[a];
+        G.Xa_after[a] = c->Xa[a];
+        G.Xb_after[a] = c->Xb[a];
     }
     for (int s = 0; s < c->nspecies; ++s) {
         G.buf_after[s] = c->sp[s].buf;
@@ -851,6 +855,9 @@ static void graph_apply_after(Ctx *c, const StepGraph &G) {
     for (int a = 0; a < 3; ++a) {
         c->J[a] = G.J_after[a];
         c->Jt[a] = G.Jt_after[a];
+        c->B[a] = G.B_after[a];
+        c->Xa[a] = G.Xa_after[a];
+        c->Xb[a] = G.Xb_after[a];
     }
     for (int s = 0; s < c->nspecies; ++s) {
         Species &S = c->sp[s];
@@ -895,6 +902,7 @@ static int step_graph(Ctx *c, bool sort, bool filter) {
     G.sort = sort;
     G.filter = filter;
     G.J0 = c->J[0];
+    G.B0 = c->B[0];
     for (int s = 0; s < c->nspecies; ++s) {
         G.buf[s] = c->sp[s].buf;
         G.sorted[s] = c->sp[s].sorted;

@@ -501,13 +501,14 @@ struct Species {
 
 // One step captured as a CUDA graph (pp_set_graphs).  A step's launches and
 // their pointer arguments are fixed by the state it starts from: whether it
-// sorts, which of J / J' holds the current, and which buffer holds each
-// species (the sort swaps them).  The host-side state the step leaves behind
+// sorts, which of J / J' holds the current, which array holds B (the field
+// update swaps it with its last iterate), and which buffer holds each species
+// (the sort swaps them).  The host-side state the step leaves behind
 // is stored with it and re-applied on every replay.
 struct StepGraph {
     bool valid = false;
     bool sort = false;
-    void *J0 = nullptr;
+    void *J0 = nullptr, *B0 = nullptr;
     void *buf[PP_MAX_SPECIES] = {};
     bool sorted[PP_MAX_SPECIES] = {};
     bool fresh[PP_MAX_SPECIES] = {};
@@ -515,7 +516,7 @@ struct StepGraph {
     cudaGraphExec_t exec = nullptr;
     int launches = 0;
     bool filter = false;
-    void *J_after[3] = {}, *Jt_after[3] = {};
+    void *J_after[3] = {}, *Jt_after[3] = {}, *B_after[3] = {}, *Xa_after[3] = {}, *Xb_after[3] = {};
     void *buf_after[PP_MAX_SPECIES] = {}, *alt_after[PP_MAX_SPECIES] = {};
     bool sorted_after[PP_MAX_SPECIES] = {}, fresh_after[PP_MAX_SPECIES] = {};
     bool pending_after[PP_MAX_SPECIES] = {}, keys_valid_after[PP_MAX_SPECIES] = {};
@@ -525,6 +526,7 @@ struct StepGraph {
     bool filtered_after_solve = false;
 };
 constexpr int kGraphSlots = 8;
+constexpr int kMaxTaps = 64;   // taps of the high-order current's line operator inverse, per axis
 
 enum Phase { PH_PARTICLE = 0, PH_CURRENT = 1, PH_FIELD = 2, PH_SORT = 3, PH_N = 4 };
 
@@ -546,7 +548,7 @@ struct Ctx {
     bool have_G0 = false;
     // high-order current: symmetric circulant taps of the inverse of the
     // (c, b+c, a+b+c, b+c, c) line operator, per axis
-    double *taps = nullptr;  // device, 3 x kMaxTaps
+    double h_taps[3 * kMaxTaps] = {};
     int ntaps[3] = {0, 0, 0};
     bool full_circ[3] = {false, false, false};
     // field solve
@@ -622,6 +624,7 @@ struct Ctx {
     int *d_status = nullptr;
     int *h_status = nullptr;     // pinned mirror
     unsigned long long *d_nslow = nullptr;
+    bool nslow_set = false;      // the last pass counted into it
     unsigned *d_slow_count = nullptr;   // per species, particles left to the global-mesh kernel
     // reductions
     double *d_red = nullptr;     // partials
@@ -638,8 +641,6 @@ struct Ctx {
     Species sp[PP_MAX_SPECIES];
     char err[512] = {0};
 };
-
-constexpr int kMaxTaps = 64;
 
 // ---------------------------------------------------------------------------
 // Kernel launchers (defined in the .cu files); all enqueue on c.st.

@@ -5,7 +5,7 @@
 //
 // Mesh arrays are padded (Geom::at).  E and B keep their periodic ghost layers
 // filled (the particle gather reads them), and so do the relaxation iterates:
-// the implicit solver's stencils read those through linear offsets (NbLin).
+// the implicit solver's stencils read those through linear offsets.
 // Other stencils read interior values through periodic wrapping (Nb).
 #include "pp_internal.cuh"
 
@@ -19,69 +19,57 @@ __device__ __forceinline__ void unflatten(int64_t t, const Geom &g, int &i, int 
 }
 
 // ---------------------------------------------------------------------------
-// Ghost fold: every interior node collects the ghost images of itself along
-// one axis (coordinate + m*n, m != 0, inside the padding) and the ghosts are
-// cleared.  Passes x, y, z in turn; each ghost is read by exactly one thread.
+// Ghost fold: every interior node near a face collects the ghost images of
+// itself (coordinates + m n inside the padding, all axes at once).  The ghosts
+// are only read, each by one thread, and keep their values: nothing reads the
+// ghosts of J (its stencils wrap), and the next pass clears the arrays.  One
+// launch over the interior, in which a node without images costs its index
+// alone; one pass per axis over all nodes, read and written, measured 0.36 ms
+// on 256 x 128 x 128 nodes of FP32, this one about 0.03 ms.
 // ---------------------------------------------------------------------------
 template <typename R>
-__global__ void k_fold_axis(Geom g, R *J0, R *J1, R *J2, int axis, int lo0, int lo1, int lo2, int e0, int e1,
-                            int e2) {
-    int64_t total = (int64_t)e0 * e1 * e2;
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= total) return;
-    int c[3];
-    c[0] = lo0 + (int)(t % e0);
-    int64_t r = t / e0;
-    c[1] = lo1 + (int)(r % e1);
-    c[2] = lo2 + (int)(r / e1);
-    R *Js[3] = {J0, J1, J2};
-    int n = g.n[axis];
-    int64_t base = g.at(c[0], c[1], c[2]);
-    int64_t stride = axis == 0 ? 1 : (axis == 1 ? (int64_t)g.P[0] : (int64_t)g.P[0] * g.P[1]);
-    int x = c[axis];
-    for (int comp = 0; comp < 3; ++comp) {
-        R *J = Js[comp];
-        R acc = J[base];
-        for (int m = -((g.G + n - 1) / n); m <= (g.G + n - 1) / n; ++m) {
-            if (m == 0) continue;
-            int y = x + m * n;
-            if (y < -g.G || y >= n + g.G) continue;
-            int64_t q = base + (int64_t)(y - x) * stride;
-            acc += J[q];
-            J[q] = R(0);
-        }
-        J[base] = acc;
+__global__ void __launch_bounds__(256) k_fold(Geom g, R *J0, R *J1, R *J2) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
+    if (i >= g.n[0] || j >= g.n[1]) return;
+    const int c[3] = {i, j, k};
+    int lo[3];   // lowest image coordinate per axis
+    bool any = false;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        lo[a] = c[a];
+        while (lo[a] - g.n[a] >= -g.G) lo[a] -= g.n[a];
+        any = any || lo[a] != c[a] || c[a] + g.n[a] < g.n[a] + g.G;
     }
+    if (!any) return;
+    R s0 = R(0), s1 = R(0), s2 = R(0);
+    for (int z = lo[2]; z < g.n[2] + g.G; z += g.n[2])
+        for (int y = lo[1]; y < g.n[1] + g.G; y += g.n[1])
+            for (int x = lo[0]; x < g.n[0] + g.G; x += g.n[0]) {
+                const int64_t q = g.at(x, y, z);
+                s0 += J0[q];
+                s1 += J1[q];
+                s2 += J2[q];
+            }
+    const int64_t q = g.at(i, j, k);
+    J0[q] = s0;
+    J1[q] = s1;
+    J2[q] = s2;
 }
 
 template <typename R>
 static cudaError_t fold_impl(Ctx &c) {
     const Geom &g = c.g;
-    int G = g.G;
-    R *J0 = (R *)c.J[0], *J1 = (R *)c.J[1], *J2 = (R *)c.J[2];
-    // x pass over padded y, z; y pass over interior x, padded z; z pass over interior x, y
-    int lo[3][3] = {{0, -G, -G}, {0, 0, -G}, {0, 0, 0}};
-    int ex[3][3] = {{g.n[0], g.n[1] + 2 * G, g.n[2] + 2 * G}, {g.n[0], g.n[1], g.n[2] + 2 * G}, {g.n[0], g.n[1], g.n[2]}};
-    for (int a = 0; a < 3; ++a) {
-        int64_t total = (int64_t)ex[a][0] * ex[a][1] * ex[a][2];
-        k_fold_axis<R><<<(unsigned)((total + 255) / 256), 256, 0, c.st>>>(g, J0, J1, J2, a, lo[a][0], lo[a][1], lo[a][2],
-                                                                          ex[a][0], ex[a][1], ex[a][2]);
-        ++c.nlaunch;
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    const dim3 b(32, 8), n((unsigned)((g.n[0] + 31) / 32), (unsigned)((g.n[1] + 7) / 8), (unsigned)g.n[2]);
+    k_fold<R><<<n, b, 0, c.st>>>(g, (R *)c.J[0], (R *)c.J[1], (R *)c.J[2]);
+    ++c.nlaunch;
+    return cudaGetLastError();
 }
 
 cudaError_t launch_fold_J(Ctx &c) { return c.fp64 ? fold_impl<double>(c) : fold_impl<float>(c); }
 
 cudaError_t launch_zero_J(Ctx &c) {
-    size_t bytes = (size_t)c.g.padded_size() * c.rsz;
-    for (int a = 0; a < 3; ++a) {
-        cudaError_t e = cudaMemsetAsync(c.J[a], 0, bytes, c.st);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    // the components of J (and of J') follow one another in the mesh allocation
+    return cudaMemsetAsync(c.J[0], 0, (size_t)c.g.padded_size() * c.rsz * 3, c.st);
 }
 
 // ---------------------------------------------------------------------------
@@ -295,50 +283,76 @@ cudaError_t launch_window_fields(Ctx &c) {
 // exact (or exponentially truncated) circulant inverse, taps precomputed in
 // FP64 on the host.  out(i) = sum_m T[m] * in(i + off + m).
 // ---------------------------------------------------------------------------
-struct TapSet {
-    const double *T[3];
-    int L[3];
-    int off[3];
+// Bound by load issue: 17 taps of FP32 values that L1 serves (a block spans 32
+// nodes along x and 8 along its component's axis, so the 8 + 16 rows it reads
+// stay there).  Taps arrive in the kernel's arguments, and only nodes within
+// the reach of a face wrap.  The previous form (a 256-node row per block, taps
+// loaded and converted from FP64, wrapped indices throughout) took 0.47 ms on
+// 256 x 128 x 128 nodes, this one about 0.1 ms.
+template <typename R>
+struct Taps {
+    R t[3][kMaxTaps];
+    int L[3];      // taps
+    int off[3];    // offset of the first
 };
 
 template <typename R>
-__global__ void k_current_solve(Geom g, TapSet ts, const R *I0, const R *I1, const R *I2, R *O0, R *O1, R *O2) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int comp = blockIdx.y;
-    if (t >= g.cells()) return;
-    int c[3];
-    unflatten(t, g, c[0], c[1], c[2]);
+__global__ void __launch_bounds__(256) k_current_solve(Geom g, const __grid_constant__ Taps<R> ts, const R *I0,
+                                                       const R *I1, const R *I2, R *O0, R *O1, R *O2, int nb0, int nb1) {
+    // blocks of component 0 and 1 (32 x 8 nodes in x and y, one z), then of
+    // component 2 (x and z, one y)
+    int b = blockIdx.x;
+    const int comp = b < nb0 ? 0 : (b < nb0 + nb1 ? 1 : 2);
+    b -= comp == 0 ? 0 : (comp == 1 ? nb0 : nb0 + nb1);
+    const int bx = (g.n[0] + 31) / 32, ea = comp == 2 ? g.n[2] : g.n[1];
+    const int by = (ea + 7) / 8;
+    const int i = (b % bx) * 32 + (threadIdx.x & 31), v = ((b / bx) % by) * 8 + (threadIdx.x >> 5), w = b / (bx * by);
+    if (i >= g.n[0] || v >= ea) return;
+    const int j = comp == 2 ? w : v, k = comp == 2 ? v : w;
     const R *in = comp == 0 ? I0 : (comp == 1 ? I1 : I2);
     R *out = comp == 0 ? O0 : (comp == 1 ? O1 : O2);
-    const double *T = ts.T[comp];
-    int L = ts.L[comp], off = ts.off[comp], n = g.n[comp];
-    int x = c[comp];
+    const int L = ts.L[comp], n = comp == 0 ? g.n[0] : ea;
+    const int stride = comp == 0 ? 1 : (comp == 1 ? g.P[0] : g.P[0] * g.P[1]);
+    const int x = comp == 0 ? i : v, x0 = x + ts.off[comp];
+    const int q = (int)g.at(i, j, k);
     R acc = R(0);
-    int q[3] = {c[0], c[1], c[2]};
-    for (int m = 0; m < L; ++m) {
-        q[comp] = wrap(x + off + m, n);
-        acc += (R)__ldg(T + m) * in[g.at(q[0], q[1], q[2])];
+    if (x0 >= 0 && x0 + L <= n) {
+        const R *p = in + q + (x0 - x) * stride;
+#pragma unroll 4
+        for (int m = 0; m < L; ++m) acc += ts.t[comp][m] * p[m * stride];
+    } else {
+        const R *p = in + q - x * stride;
+        int y = x0;
+#pragma unroll 4
+        for (int m = 0; m < L; ++m, ++y) acc += ts.t[comp][m] * p[(y < 0 ? y + n : (y >= n ? y - n : y)) * stride];
     }
-    out[g.at(c[0], c[1], c[2])] = acc;
+    out[q] = acc;
+}
+
+template <typename R>
+static cudaError_t current_solve_impl(Ctx &c) {
+    const Geom &g = c.g;
+    Taps<R> ts;
+    for (int a = 0; a < 3; ++a) {
+        const int n = c.ntaps[a];
+        for (int m = 0; m < kMaxTaps; ++m) ts.t[a][m] = m < n ? (R)c.h_taps[a * kMaxTaps + m] : R(0);
+        ts.L[a] = n;
+        ts.off[a] = -(n / 2);
+        if (c.full_circ[a])   // the whole period: rotate so that it starts n / 2 below the node
+            for (int m = 0; m < n; ++m) ts.t[a][m] = (R)c.h_taps[a * kMaxTaps + (m + n - n / 2) % n];
+    }
+    const int64_t bx = (g.n[0] + 31) / 32;
+    const int64_t xy = bx * ((g.n[1] + 7) / 8) * g.n[2], xz = bx * ((g.n[2] + 7) / 8) * g.n[1];
+    k_current_solve<R><<<(unsigned)(2 * xy + xz), 256, 0, c.st>>>(
+        g, ts, (const R *)c.J[0], (const R *)c.J[1], (const R *)c.J[2], (R *)c.Jt[0], (R *)c.Jt[1], (R *)c.Jt[2], (int)xy,
+        (int)xy);
+    ++c.nlaunch;
+    return cudaGetLastError();
 }
 
 cudaError_t launch_current_solve(Ctx &c) {
     if (c.d.field_order == 2) return cudaSuccess;
-    TapSet ts;
-    for (int a = 0; a < 3; ++a) {
-        ts.T[a] = c.taps + a * kMaxTaps;
-        ts.L[a] = c.ntaps[a];
-        ts.off[a] = c.full_circ[a] ? 0 : -(c.ntaps[a] / 2);
-    }
-    dim3 grid((unsigned)((c.g.cells() + 255) / 256), 3);
-    if (c.fp64)
-        k_current_solve<double><<<grid, 256, 0, c.st>>>(c.g, ts, (double *)c.J[0], (double *)c.J[1], (double *)c.J[2],
-                                                        (double *)c.Jt[0], (double *)c.Jt[1], (double *)c.Jt[2]);
-    else
-        k_current_solve<float><<<grid, 256, 0, c.st>>>(c.g, ts, (float *)c.J[0], (float *)c.J[1], (float *)c.J[2],
-                                                       (float *)c.Jt[0], (float *)c.Jt[1], (float *)c.Jt[2]);
-    ++c.nlaunch;
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = c.fp64 ? current_solve_impl<double>(c) : current_solve_impl<float>(c);
     if (e != cudaSuccess) return e;
     for (int a = 0; a < 3; ++a) {
         void *t = c.J[a];
@@ -401,47 +415,8 @@ struct Vec3 {
     const R *p[3];
 };
 
-// Neighbours by linear offsets into a padded array whose periodic ghost
-// layers (width kGhost >= the stencil reach 5) hold valid images: no index
-// wrapping.  Same stencils as Nb.
-template <typename R>
-struct NbLin {
-    int64_t q;      // padded index of the cell
-    int64_t s[3];   // strides of x, y, z
-    __device__ __forceinline__ R at(const R *f, int axis, int o) const { return f[q + o * s[axis]]; }
-    __device__ __forceinline__ R dplus(const R *f, int axis, const FieldCoef &k) const {
-        R v = R(0);
-#pragma unroll
-        for (int m = 1; m <= 3; ++m) v += (R)k.k[m - 1] * (at(f, axis, m) - at(f, axis, 1 - m));
-        return v * (R)k.ih[axis];
-    }
-    __device__ __forceinline__ R dminus(const R *f, int axis, const FieldCoef &k) const {
-        R v = R(0);
-#pragma unroll
-        for (int m = 1; m <= 3; ++m) v += (R)k.k[m - 1] * (at(f, axis, m - 1) - at(f, axis, -m));
-        return v * (R)k.ih[axis];
-    }
-    __device__ __forceinline__ R lap(const R *f, const FieldCoef &k) const {
-        R center = f[q];
-        R v = R(0);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            R sa = (R)k.lap[0] * center;
-#pragma unroll
-            for (int o = 1; o <= 5; ++o) sa += (R)k.lap[o] * (at(f, a, o) + at(f, a, -o));
-            v += sa * (R)k.ih2[a];
-        }
-        return v;
-    }
-};
-
-template <typename R>
-__device__ __forceinline__ NbLin<R> nb_lin(const Geom &g, int i, int j, int k) {
-    return NbLin<R>{g.at(i, j, k), {1, (int64_t)g.P[0], (int64_t)g.P[0] * g.P[1]}};
-}
-
 // Store v at interior cell (i, j, k) and at every periodic image of it inside
-// the ghost layers, so that the array stays readable through NbLin.  Every
+// the ghost layers, so that the array stays readable by linear offsets.  Every
 // ghost cell is the image of exactly one interior cell.
 template <typename R>
 __device__ __forceinline__ void store_periodic(R *f, const Geom &g, int i, int j, int k, R v) {
@@ -452,13 +427,6 @@ __device__ __forceinline__ void store_periodic(R *f, const Geom &g, int i, int j
     for (int z = z0; z < g.n[2] + g.G; z += g.n[2])
         for (int y = y0; y < g.n[1] + g.G; y += g.n[1])
             for (int x = x0; x < g.n[0] + g.G; x += g.n[0]) f[g.at(x, y, z)] = v;
-}
-
-// Launch shape of the cell kernels below: x along threads, y and z along the
-// grid (no division to recover the cell).
-constexpr int kCellThreads = 128;
-static inline dim3 cell_grid(const Geom &g) {
-    return dim3((unsigned)((g.n[0] + kCellThreads - 1) / kCellThreads), (unsigned)g.n[1], (unsigned)g.n[2]);
 }
 
 // rhs_a = B_a + alpha beta dt^2 (L B)_a - dt (curl^+ E)_a + alpha dt^2 (curl^+ J)_a
@@ -481,154 +449,245 @@ __global__ void k_rhs(Geom g, FieldCoef k, Vec3<R> E, Vec3<R> B, Vec3<R> J, R *O
     }
 }
 
-// k_rhs for B and E with valid ghost layers (the implicit solver): B and E
-// through linear offsets, J (ghosts cleared by the fold) through wrapping.
+// ---- the implicit solver's kernels: W nodes along x per thread ----
+// B and E arrive with valid ghost layers and every kernel that writes them here
+// writes their images too, so stencils read through linear offsets and no pass
+// copies ghosts.  With an even mesh size along x (rows of an even number of
+// nodes, the interior starting at an even one) W = 2: every value along y and
+// z is one aligned pair load, and a pair's row of x neighbours six or seven.
+// Nothing is staged in shared memory and no barrier joins the threads: L1
+// holds the rows that a block's 32 x 8 threads share.
 template <typename R>
-__global__ void k_rhs_lin(Geom g, FieldCoef k, Vec3<R> E, Vec3<R> B, Vec3<R> J, R *O0, R *O1, R *O2, R ab_dt2,
-                          R dt, R a_dt2) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= g.n[0]) return;
-    int j = blockIdx.y, kz = blockIdx.z;
-    NbLin<R> nl = nb_lin<R>(g, i, j, kz);
-    Nb<R> nb{g, {i, j, kz}};
-    R *out[3] = {O0, O1, O2};
+struct Coef {
+    R k[3], lap[6], ih[3], ih2[3];
+};
+template <typename R, int W>
+struct Nodes {
+    R v[W];
+};
+template <int W, typename R>
+__device__ __forceinline__ Nodes<R, W> ld(const R *p) {
+    Nodes<R, W> r;
+    if constexpr (W == 1) {
+        r.v[0] = *p;
+    } else if constexpr (sizeof(R) == 4) {
+        const float2 t = *reinterpret_cast<const float2 *>(p);
+        r.v[0] = t.x;
+        r.v[1] = t.y;
+    } else {
+        const double2 t = *reinterpret_cast<const double2 *>(p);
+        r.v[0] = t.x;
+        r.v[1] = t.y;
+    }
+    return r;
+}
+
+// The row of x neighbours from node -N (N even for W = 2) to node N + W - 1 of
+// the thread's nodes; the thread's own are given.
+template <int N, typename R, int W>
+struct Row {
+    R v[2 * N + W];
+    __device__ __forceinline__ Row(const R *p) {
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const int b = (a + 1) % 3, c = (a + 2) % 3;
-        R curlE = nl.dplus(E.p[c], b, k) - nl.dplus(E.p[b], c, k);
-        R curlJ = nb.dplus(J.p[c], b, k) - nb.dplus(J.p[b], c, k);
-        out[a][nl.q] = B.p[a][nl.q] + ab_dt2 * nl.lap(B.p[a], k) - dt * curlE + a_dt2 * curlJ;
+        for (int m = 0; m < 2 * N + W; m += W) {
+            const Nodes<R, W> t = ld<W>(p + m - N);
+#pragma unroll
+            for (int w = 0; w < W; ++w) v[m + w] = t.v[w];
+        }
+    }
+    __device__ __forceinline__ R at(int o, int w) const { return v[N + o + w]; }
+};
+template <int W>
+constexpr int even(int n) {
+    return W == 2 ? (n + 1) / 2 * 2 : n;
+}
+
+// d^+ (plus) or d^- of f along `axis` at the thread's nodes.
+template <typename R, int W>
+__device__ __forceinline__ Nodes<R, W> diff(const R *f, int axis, int stride, bool plus, const Coef<R> &k) {
+    Nodes<R, W> r;
+#pragma unroll
+    for (int w = 0; w < W; ++w) r.v[w] = R(0);
+    if (axis == 0) {
+        const Row<even<W>(3), R, W> x(f);
+#pragma unroll
+        for (int m = 1; m <= 3; ++m)
+#pragma unroll
+            for (int w = 0; w < W; ++w) r.v[w] += k.k[m - 1] * (plus ? x.at(m, w) - x.at(1 - m, w) : x.at(m - 1, w) - x.at(-m, w));
+    } else {
+#pragma unroll
+        for (int m = 1; m <= 3; ++m) {
+            const Nodes<R, W> u = ld<W>(f + (plus ? m : m - 1) * stride), d = ld<W>(f + (plus ? 1 - m : -m) * stride);
+#pragma unroll
+            for (int w = 0; w < W; ++w) r.v[w] += k.k[m - 1] * (u.v[w] - d.v[w]);
+        }
+    }
+#pragma unroll
+    for (int w = 0; w < W; ++w) r.v[w] *= k.ih[axis];
+    return r;
+}
+
+// d^+ of J, whose ghosts are not valid: the thread's nodes wrap.  x: the
+// nodes' coordinate along the axis, n its size.
+template <typename R, int W>
+__device__ __forceinline__ Nodes<R, W> diff_wrap(const R *f, int axis, int stride, int x, int n, const Coef<R> &k) {
+    Nodes<R, W> r;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        R s = R(0);
+        const int c = axis == 0 ? x + w : x;
+#pragma unroll
+        for (int m = 1; m <= 3; ++m)
+            s += k.k[m - 1] * (f[w + (wrap(c + m, n) - c) * stride] - f[w + (wrap(c + 1 - m, n) - c) * stride]);
+        r.v[w] = s * k.ih[axis];
+    }
+    return r;
+}
+
+// L f at the thread's nodes: per axis the symmetric 11-point stencil.
+// col: the 11 nodes along z.
+template <typename R, int W>
+__device__ __forceinline__ Nodes<R, W> laplace(const R *f, int sy, const Nodes<R, W> (&col)[11], const Coef<R> &k) {
+    Nodes<R, W> r, s;
+    const Row<even<W>(5), R, W> x(f);
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        s.v[w] = k.lap[0] * col[5].v[w];
+#pragma unroll
+        for (int o = 1; o <= 5; ++o) s.v[w] += k.lap[o] * (x.at(o, w) + x.at(-o, w));
+        r.v[w] = s.v[w] * k.ih2[0];
+        s.v[w] = k.lap[0] * col[5].v[w];
+    }
+#pragma unroll
+    for (int o = 1; o <= 5; ++o) {
+        const Nodes<R, W> u = ld<W>(f + o * sy), d = ld<W>(f - o * sy);
+#pragma unroll
+        for (int w = 0; w < W; ++w) s.v[w] += k.lap[o] * (u.v[w] + d.v[w]);
+    }
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        r.v[w] += s.v[w] * k.ih2[1];
+        s.v[w] = k.lap[0] * col[5].v[w];
+#pragma unroll
+        for (int o = 1; o <= 5; ++o) s.v[w] += k.lap[o] * (col[5 + o].v[w] + col[5 - o].v[w]);
+        r.v[w] += s.v[w] * k.ih2[2];
+    }
+    return r;
+}
+
+// Store the thread's nodes (i, j, z) and their periodic images.
+template <typename R, int W>
+__device__ __forceinline__ void store_nodes(R *f, const Geom &g, int q, int i, int j, int z, const Nodes<R, W> &v) {
+    const bool inner = i >= g.G && i + W <= g.n[0] - g.G && j >= g.G && j < g.n[1] - g.G && z >= g.G && z < g.n[2] - g.G;
+    if (inner) {
+        if constexpr (W == 1) f[q] = v.v[0];
+        else if constexpr (sizeof(R) == 4) *reinterpret_cast<float2 *>(f + q) = make_float2(v.v[0], v.v[1]);
+        else *reinterpret_cast<double2 *>(f + q) = make_double2(v.v[0], v.v[1]);
+    } else {
+#pragma unroll
+        for (int w = 0; w < W; ++w) store_periodic(f, g, i + w, j, z, v.v[w]);
     }
 }
 
-// One Chebyshev sweep (Saad's three-term form, see field_update_impl), plane by
-// plane: r = rhs - X + kk L X, X_new = X + c1 (X - X_prev) + c2 r, with each
-// component's 31-point Laplacian (NbLin::lap, the same sums in the same order) read
-// from a shared xy plane (the block's 32 x 8 nodes and 5 nodes of halo on each
-// side) and a register column of the 11 z nodes around the plane.  A block
-// marches through kChebZ planes of one component, so every node of X comes
-// from L2 or HBM about three times (column, halo, chunk start) instead of 31.
-// Planes per block: 8 measured best (C3 beam field update 2.62 ms per step
-// against 2.68 at 16 and 2.91 at 32; 3.80 for the node-per-thread sweep that
-// read every neighbour through L1/L2).
-#ifndef PP_CHEB_Z
-#define PP_CHEB_Z 8
-#endif
-constexpr int kChebBX = 32, kChebBY = 8, kChebZ = PP_CHEB_Z, kChebR = 5;
-
 template <typename R>
-__global__ void __launch_bounds__(kChebBX *kChebBY) k_cheb_plane(Geom g, FieldCoef k, Vec3<R> X, Vec3<R> Xp, Vec3<R> Rh,
-                                                                 R *O0, R *O1, R *O2, R kk, R c1, R c2, int nzc) {
-    __shared__ R pl[kChebBY + 2 * kChebR][kChebBX + 2 * kChebR];
-    const int tx = threadIdx.x % kChebBX, ty = threadIdx.x / kChebBX;
-    const int x0 = blockIdx.x * kChebBX, y0 = blockIdx.y * kChebBY;
-    const int a = blockIdx.z / nzc, zc = blockIdx.z - a * nzc;
-    const int z0 = zc * kChebZ, z1 = min(g.n[2], z0 + kChebZ);
-    const int i = x0 + tx, j = y0 + ty;
-    const bool mine = i < g.n[0] && j < g.n[1];
-    // the component's arrays, selected without indexing the parameter arrays
-    // at run time (which would copy them to local memory)
-    const R *f = a == 0 ? X.p[0] : (a == 1 ? X.p[1] : X.p[2]);
-    const R *fp = a == 0 ? Xp.p[0] : (a == 1 ? Xp.p[1] : Xp.p[2]);
-    const R *rh = a == 0 ? Rh.p[0] : (a == 1 ? Rh.p[1] : Rh.p[2]);
+__device__ __forceinline__ const R *pick(const Vec3<R> &v, int a) {   // no run-time index into the arguments
+    return a == 0 ? v.p[0] : (a == 1 ? v.p[1] : v.p[2]);
+}
+
+// rhs_a = B_a + alpha beta dt^2 (L B)_a - dt (curl^+ E)_a + alpha dt^2 (curl^+ J)_a
+template <typename R, int W>
+__global__ void __launch_bounds__(256) k_rhs_lin(Geom g, const __grid_constant__ Coef<R> k, Vec3<R> E, Vec3<R> B,
+                                                 Vec3<R> J, R *O0, R *O1, R *O2, R ab_dt2, R dt, R a_dt2) {
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) * W, j = blockIdx.y * blockDim.y + threadIdx.y;
+    if (i >= g.n[0] || j >= g.n[1]) return;
+    const int z = blockIdx.z % g.n[2], a = blockIdx.z / g.n[2];
+    const int b = a == 2 ? 0 : a + 1, c = a == 0 ? 2 : a - 1;
+    const int sy = g.P[0], sz = g.P[0] * g.P[1];
+    const int q = (int)g.at(i, j, z);
+    const R *f = pick(B, a) + q;
+    Nodes<R, W> col[11];
+#pragma unroll
+    for (int m = 0; m < 11; ++m) col[m] = ld<W>(f + (m - 5) * sz);
+    const Nodes<R, W> L = laplace<R, W>(f, sy, col, k);
+    const int sb = b == 0 ? 1 : (b == 1 ? sy : sz), sc = c == 0 ? 1 : (c == 1 ? sy : sz);
+    // curl_a = d_b F_c - d_c F_b
+    const Nodes<R, W> e1 = diff<R, W>(pick(E, c) + q, b, sb, true, k), e2 = diff<R, W>(pick(E, b) + q, c, sc, true, k);
+    Nodes<R, W> j1, j2;
+    if (i >= 2 && i + W + 2 < g.n[0] && j >= 2 && j + 3 < g.n[1] && z >= 2 && z + 3 < g.n[2]) {
+        j1 = diff<R, W>(pick(J, c) + q, b, sb, true, k);
+        j2 = diff<R, W>(pick(J, b) + q, c, sc, true, k);
+    } else {
+        const int xb = b == 0 ? i : (b == 1 ? j : z), xc = c == 0 ? i : (c == 1 ? j : z);
+        const int nb = b == 0 ? g.n[0] : (b == 1 ? g.n[1] : g.n[2]), nc = c == 0 ? g.n[0] : (c == 1 ? g.n[1] : g.n[2]);
+        j1 = diff_wrap<R, W>(pick(J, c) + q, b, sb, xb, nb, k);
+        j2 = diff_wrap<R, W>(pick(J, b) + q, c, sc, xc, nc, k);
+    }
     R *out = a == 0 ? O0 : (a == 1 ? O1 : O2);
-    // Each thread reads at most five x, y positions of the padded array (its
-    // column and up to four halo nodes); their plane-0 offsets and whether
-    // they lie inside the padded array (every node a computed node reads
-    // does) are fixed for the whole march.
-    const int64_t ps = (int64_t)g.P[0] * g.P[1];
-    auto inside = [&](int x, int y) { return x >= -g.G && x < g.n[0] + g.G && y >= -g.G && y < g.n[1] + g.G; };
-    const bool okc = inside(i, j);
-    const int64_t qc = okc ? g.at(i, j, 0) : 0;
-    const bool okx0 = tx < kChebR && inside(x0 + tx - kChebR, j), okx1 = tx < kChebR && inside(x0 + kChebBX + tx, j);
-    const bool oky0 = ty < kChebR && inside(i, y0 + ty - kChebR), oky1 = ty < kChebR && inside(i, y0 + kChebBY + ty);
-    const int64_t qx0 = okx0 ? g.at(x0 + tx - kChebR, j, 0) : 0, qx1 = okx1 ? g.at(x0 + kChebBX + tx, j, 0) : 0;
-    const int64_t qy0 = oky0 ? g.at(i, y0 + ty - kChebR, 0) : 0, qy1 = oky1 ? g.at(i, y0 + kChebBY + ty, 0) : 0;
-    // no periodic image of this column's nodes inside the ghost layers on x or y
-    const bool noimg_xy = i >= g.G && i < g.n[0] - g.G && j >= g.G && j < g.n[1] - g.G;
-    R col[2 * kChebR + 1];
 #pragma unroll
-    for (int m = 0; m < 2 * kChebR + 1; ++m) col[m] = okc ? f[qc + (int64_t)(z0 - kChebR + m) * ps] : R(0);
-    R lp[kChebR + 1];
+    for (int w = 0; w < W; ++w)
+        out[q + w] = col[5].v[w] + ab_dt2 * L.v[w] - dt * (e1.v[w] - e2.v[w]) + a_dt2 * (j1.v[w] - j2.v[w]);
+}
+
+// One Chebyshev sweep (Saad's three-term form, see field_update_impl):
+// r = rhs - X + kk L X, X_new = X + c1 (X - X_prev) + c2 r.  A thread marches
+// through zper planes of one component with the 11 nodes along z in registers.
+// FP32 on large meshes: bound by the L1 and L2 traffic of the neighbours;
+// FP64: by the part's FP64 rate (about 40 operations a node and component);
+// small meshes: by launch and load latency, so the march is cut until every
+// SM has threads.  CHEB_FIG
+template <typename R, int W>
+__global__ void __launch_bounds__(256) k_cheb(Geom g, const __grid_constant__ Coef<R> k, Vec3<R> X, Vec3<R> Xp,
+                                              Vec3<R> Rh, R *O0, R *O1, R *O2, R kk, R c1, R c2, int zper, int nzc) {
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) * W, j = blockIdx.y * blockDim.y + threadIdx.y;
+    if (i >= g.n[0] || j >= g.n[1]) return;
+    const int a = blockIdx.z / nzc, z0 = (blockIdx.z - a * nzc) * zper, z1 = min(g.n[2], z0 + zper);
+    const int sy = g.P[0], sz = g.P[0] * g.P[1];
+    int q = (int)g.at(i, j, z0);
+    const R *f = pick(X, a), *fp = pick(Xp, a), *rh = pick(Rh, a);
+    R *out = a == 0 ? O0 : (a == 1 ? O1 : O2);
+    Nodes<R, W> col[11];
 #pragma unroll
-    for (int o = 0; o <= kChebR; ++o) lp[o] = (R)k.lap[o];
-    const R ih2x = (R)k.ih2[0], ih2y = (R)k.ih2[1], ih2z = (R)k.ih2[2];
-    // the next plane's halo nodes, rhs and previous iterate are loaded one
-    // plane ahead, so that their latency overlaps the current plane's work
-    R hx0 = R(0), hx1 = R(0), hy0 = R(0), hy1 = R(0), rhn = R(0), xpn = R(0);
-    auto fetch = [&](int z) {
-        const int64_t zo = (int64_t)z * ps;
-        if (okx0) hx0 = f[qx0 + zo];
-        if (okx1) hx1 = f[qx1 + zo];
-        if (oky0) hy0 = f[qy0 + zo];
-        if (oky1) hy1 = f[qy1 + zo];
-        if (mine) {
-            rhn = rh[qc + zo];
-            xpn = fp[qc + zo];
+    for (int m = 0; m < 11; ++m) col[m] = ld<W>(f + q + (m - 5) * sz);
+    for (int z = z0;;) {
+        const Nodes<R, W> xp = ld<W>(fp + q), rz = ld<W>(rh + q);
+        const Nodes<R, W> L = laplace<R, W>(f + q, sy, col, k);
+        Nodes<R, W> nv;
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            const R x = col[5].v[w];
+            const R r = rz.v[w] - x + kk * L.v[w];
+            nv.v[w] = x + c1 * (x - xp.v[w]) + c2 * r;
         }
-    };
-    fetch(z0);
-    for (int z = z0; z < z1; ++z) {
-        pl[ty + kChebR][tx + kChebR] = col[kChebR];
-        if (tx < kChebR) {
-            pl[ty + kChebR][tx] = hx0;
-            pl[ty + kChebR][tx + kChebBX + kChebR] = hx1;
-        }
-        if (ty < kChebR) {
-            pl[ty][tx + kChebR] = hy0;
-            pl[ty + kChebBY + kChebR][tx + kChebR] = hy1;
-        }
-        const R rhz = rhn, xpz = xpn;
-        __syncthreads();
-        if (z + 1 < z1) fetch(z + 1);
-        if (mine) {
-            const R center = col[kChebR];
-            R v = R(0);
-            R sa = lp[0] * center;
+        store_nodes<R, W>(out, g, q, i, j, z, nv);
+        if (++z >= z1) break;
+        q += sz;
 #pragma unroll
-            for (int o = 1; o <= kChebR; ++o)
-                sa += lp[o] * (pl[ty + kChebR][tx + kChebR + o] + pl[ty + kChebR][tx + kChebR - o]);
-            v += sa * ih2x;
-            sa = lp[0] * center;
-#pragma unroll
-            for (int o = 1; o <= kChebR; ++o)
-                sa += lp[o] * (pl[ty + kChebR + o][tx + kChebR] + pl[ty + kChebR - o][tx + kChebR]);
-            v += sa * ih2y;
-            sa = lp[0] * center;
-#pragma unroll
-            for (int o = 1; o <= kChebR; ++o) sa += lp[o] * (col[kChebR + o] + col[kChebR - o]);
-            v += sa * ih2z;
-            const R x = center;
-            const R r = rhz - x + kk * v;
-            const R nv = x + c1 * (x - xpz) + c2 * r;
-            if (noimg_xy && z >= g.G && z < g.n[2] - g.G)
-                out[qc + (int64_t)z * ps] = nv;
-            else
-                store_periodic(out, g, i, j, z, nv);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int m = 0; m < 2 * kChebR; ++m) col[m] = col[m + 1];
-        if (z + 1 < z1 && okc) col[2 * kChebR] = f[qc + (int64_t)(z + 1 + kChebR) * ps];
+        for (int m = 0; m < 10; ++m) col[m] = col[m + 1];
+        col[10] = ld<W>(f + q + 5 * sz);
     }
 }
 
-// k_e_update with Bn and Bo ghost-valid (linear offsets).
-template <typename R>
-__global__ void k_e_update_lin(Geom g, FieldCoef k, R *E0, R *E1, R *E2, Vec3<R> Bn, Vec3<R> Bo, Vec3<R> J, R alpha,
-                               R beta, R dt) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= g.n[0]) return;
-    int j = blockIdx.y, kz = blockIdx.z;
-    NbLin<R> nl = nb_lin<R>(g, i, j, kz);
-    R *E[3] = {E0, E1, E2};
+// E_new = E + dt (curl^- (alpha B_new + beta B_old) - J), ghosts of E included.
+// E is read at the thread's own nodes only, so it is updated in place.
+template <typename R, int W>
+__global__ void __launch_bounds__(256) k_e_update_lin(Geom g, const __grid_constant__ Coef<R> k, R *E0, R *E1, R *E2,
+                                                      Vec3<R> Bn, Vec3<R> Bo, Vec3<R> J, R alpha, R beta, R dt) {
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) * W, j = blockIdx.y * blockDim.y + threadIdx.y;
+    if (i >= g.n[0] || j >= g.n[1]) return;
+    const int z = blockIdx.z % g.n[2], a = blockIdx.z / g.n[2];
+    const int b = a == 2 ? 0 : a + 1, c = a == 0 ? 2 : a - 1;
+    const int sy = g.P[0], sz = g.P[0] * g.P[1];
+    const int sb = b == 0 ? 1 : (b == 1 ? sy : sz), sc = c == 0 ? 1 : (c == 1 ? sy : sz);
+    const int q = (int)g.at(i, j, z);
+    const Nodes<R, W> n1 = diff<R, W>(pick(Bn, c) + q, b, sb, false, k), n2 = diff<R, W>(pick(Bn, b) + q, c, sc, false, k);
+    const Nodes<R, W> o1 = diff<R, W>(pick(Bo, c) + q, b, sb, false, k), o2 = diff<R, W>(pick(Bo, b) + q, c, sc, false, k);
+    const Nodes<R, W> cur = ld<W>(pick(J, a) + q);
+    R *E = a == 0 ? E0 : (a == 1 ? E1 : E2);
+    Nodes<R, W> e = ld<W>((const R *)E + q);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const int b = (a + 1) % 3, c = (a + 2) % 3;
-        R cur = alpha * (nl.dminus(Bn.p[c], b, k) - nl.dminus(Bn.p[b], c, k)) +
-                beta * (nl.dminus(Bo.p[c], b, k) - nl.dminus(Bo.p[b], c, k));
-        E[a][nl.q] = E[a][nl.q] + dt * (cur - J.p[a][nl.q]);
-    }
+    for (int w = 0; w < W; ++w)
+        e.v[w] += dt * (alpha * (n1.v[w] - n2.v[w]) + beta * (o1.v[w] - o2.v[w]) - cur.v[w]);
+    store_nodes<R, W>(E, g, q, i, j, z, e);
 }
 
 // E_new = E + dt (curl^- (alpha B_new + beta B_old) - J)   (eq:enplus1, c^2 mu0 = 1)
@@ -695,28 +754,48 @@ static FieldCoef field_coef(const Ctx &c) {
 }
 
 template <typename R>
+static Coef<R> coef_of(const FieldCoef &k) {
+    Coef<R> r;
+    for (int m = 0; m < 3; ++m) {
+        r.k[m] = (R)k.k[m];
+        r.ih[m] = (R)k.ih[m];
+        r.ih2[m] = (R)k.ih2[m];
+    }
+    for (int m = 0; m < 6; ++m) r.lap[m] = (R)k.lap[m];
+    return r;
+}
+
+// Planes a thread marches through: as many as leave kMarchBlocks blocks.  A
+// march of zper planes reads zper + 10 of them.
+constexpr int kMarchBlocks = 912;
+
+template <typename R, int W>
 static cudaError_t field_update_impl(Ctx &c) {
     const Geom &g = c.g;
-    FieldCoef k = field_coef(c);
+    const Coef<R> k = coef_of<R>(field_coef(c));
     // dt of this solve: the step, or the drift of a 4th-order substep
     double al = c.d.alpha, be = 1.0 - c.d.alpha, dt = c.drift_dt;
     double kk = al * al * dt * dt;
     const Ctx::Cheb &ch = c.cheb[c.cheb_sel];
     cudaError_t e;
-    // B and E arrive with valid ghost layers (every writer of them fills
-    // them), and each sweep writes its iterate with ghosts: the stencils read
-    // through linear offsets.
-    const dim3 cg = cell_grid(g);
-    k_rhs_lin<R><<<cg, kCellThreads, 0, c.st>>>(g, k, v3<R>(c.E), v3<R>(c.B), v3<R>(c.J), (R *)c.R[0], (R *)c.R[1],
-                                                (R *)c.R[2], (R)(al * be * dt * dt), (R)dt, (R)(al * dt * dt));
+    // blocks of 256 threads (64 for FP64, whose rate wants every SM busy), as wide
+    // along x as the rows need
+    const int nx = (g.n[0] + W - 1) / W, threads = sizeof(R) == 8 ? 64 : 256;
+    int bx = 8;
+    while (bx < 32 && bx < nx) bx *= 2;
+    const dim3 blk((unsigned)bx, (unsigned)(threads / bx));
+    dim3 grid((unsigned)((nx + bx - 1) / bx), (unsigned)((g.n[1] + blk.y - 1) / blk.y), (unsigned)(3 * g.n[2]));
+    k_rhs_lin<R, W><<<grid, blk, 0, c.st>>>(g, k, v3<R>(c.E), v3<R>(c.B), v3<R>(c.J), (R *)c.R[0], (R *)c.R[1],
+                                            (R *)c.R[2], (R)(al * be * dt * dt), (R)dt, (R)(al * dt * dt));
     ++c.nlaunch;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // Chebyshev semi-iteration on the spectrum [1, lmax] of the SPD operator,
     // starting from B^n (Saad, Iterative Methods, Alg. 12.1 in 3-term form).
     double theta = ch.theta, delta = ch.delta;
-    const int nzc = (g.n[2] + kChebZ - 1) / kChebZ;
-    const dim3 pg((unsigned)((g.n[0] + kChebBX - 1) / kChebBX), (unsigned)((g.n[1] + kChebBY - 1) / kChebBY),
-                  (unsigned)(3 * nzc));
+    int zper = 16;
+    while (zper > 1 && (int64_t)grid.x * grid.y * 3 * ((g.n[2] + zper - 1) / zper) < kMarchBlocks) zper /= 2;
+    const int nzc = (g.n[2] + zper - 1) / zper;
+    const dim3 pg(grid.x, grid.y, (unsigned)(3 * nzc));
     void **cur = c.B, **prev = c.B;
     void **bufs[2] = {c.Xa, c.Xb};
     int nb = 0;
@@ -736,9 +815,8 @@ static cudaError_t field_update_impl(Ctx &c) {
         // output: a scratch buffer that is neither cur nor (when prev is B) B
         void **out = (prev == c.B || prev == cur) ? bufs[nb] : prev;
         if (out == cur) out = bufs[1 - nb];
-        k_cheb_plane<R><<<pg, kChebBX * kChebBY, 0, c.st>>>(g, k, v3<R>(cur), v3<R>(prev), v3<R>(c.R),
-                                                             (R *)out[0], (R *)out[1], (R *)out[2], (R)kk, (R)c1,
-                                                             (R)c2, nzc);
+        k_cheb<R, W><<<pg, blk, 0, c.st>>>(g, k, v3<R>(cur), v3<R>(prev), v3<R>(c.R), (R *)out[0], (R *)out[1],
+                                           (R *)out[2], (R)kk, (R)c1, (R)c2, zper, nzc);
         ++c.nlaunch;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         prev = cur;
@@ -749,16 +827,17 @@ static cudaError_t field_update_impl(Ctx &c) {
     c.last_kk = kk;
     c.filtered_after_solve = false;
     // eq:enplus1 with B^{n+1} = cur, B^n = B
-    k_e_update_lin<R><<<cg, kCellThreads, 0, c.st>>>(g, k, (R *)c.E[0], (R *)c.E[1], (R *)c.E[2], v3<R>(cur),
-                                                     v3<R>(c.B), v3<R>(c.J), (R)al, (R)be, (R)dt);
+    k_e_update_lin<R, W><<<grid, blk, 0, c.st>>>(g, k, (R *)c.E[0], (R *)c.E[1], (R *)c.E[2], v3<R>(cur), v3<R>(c.B),
+                                                 v3<R>(c.J), (R)al, (R)be, (R)dt);
     ++c.nlaunch;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    unsigned pblocks = (unsigned)((g.padded_size() + 255) / 256);
-    k_ghost_fill<R><<<pblocks, 256, 0, c.st>>>(g, (R *)c.E[0], (R *)c.E[1], (R *)c.E[2], (const R *)cur[0],
-                                               (const R *)cur[1], (const R *)cur[2], (R *)c.B[0], (R *)c.B[1],
-                                               (R *)c.B[2], 1);
-    ++c.nlaunch;
-    return cudaGetLastError();
+    // the last iterate, ghosts and all, becomes B; the old B joins the scratch
+    for (int a = 0; a < 3 && cur != c.B; ++a) {
+        void *t = c.B[a];
+        c.B[a] = cur[a];
+        cur[a] = t;
+    }
+    return cudaSuccess;
 }
 
 // Explicit FDTD variant (the cold-beam comparison of Sec. VIII): Yee's
@@ -870,7 +949,8 @@ cudaError_t launch_divergence_filter(Ctx &c) {
 cudaError_t launch_field_update(Ctx &c) {
     if (c.field_solver == PP_FIELD_EXPLICIT)
         return c.fp64 ? field_update_explicit_impl<double>(c) : field_update_explicit_impl<float>(c);
-    return c.fp64 ? field_update_impl<double>(c) : field_update_impl<float>(c);
+    if (c.g.n[0] % 2 == 0) return c.fp64 ? field_update_impl<double, 2>(c) : field_update_impl<float, 2>(c);
+    return c.fp64 ? field_update_impl<double, 1>(c) : field_update_impl<float, 1>(c);
 }
 
 template <typename R>
