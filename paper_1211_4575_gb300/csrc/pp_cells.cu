@@ -13,11 +13,14 @@
 // particles of one species:
 //
 //  phase 1, one thread per particle (a warp on 32 consecutive particles, i.e.
-//    one or two cells: the gather's shared loads are broadcasts): gather
-//    (eq:pfields), push (Vay / Boris, optional radiative cooling), move; the
-//    new cell, offset and momentum go straight back to the particle arrays
-//    (coalesced); the old offset and the displacement are staged for the
-//    deposit.  A particle whose support start changes on some axis (it
+//    one or two cells): gather (eq:pfields), push (Vay / Boris, optional
+//    radiative cooling), move; the new cell, offset and momentum go straight
+//    back to the particle arrays (coalesced); the old offset and the
+//    displacement are staged for the deposit.  The chunk passes through the
+//    tile two planes of cells at a time, whose window is expanded into pairs
+//    of neighbours along x: the gather is 192 broadcast 8-byte loads and 258
+//    packed FMAs for a PCS particle (384 4-byte loads and 504 scalar FMAs
+//    node by node).  A particle whose support start changes on some axis (it
 //    crosses a support boundary) is queued, with the axis and direction of
 //    the change.
 //  pieces: the chunk is cut into pieces of at most 8 consecutive particles
@@ -42,6 +45,11 @@
 // overflow, and after the chunk the nodes its cells reach are added into the
 // FP32 mesh (one global atomic per nonzero node).  A piece's sum is FP32 in
 // registers and is rounded to the unit once.
+//
+// Bound by issue and by the shared-memory pipe behind it: 67 warp-instructions
+// a particle at 50 % of the issue slots (64^3 thermal PCS, 16.8 M particles:
+// 2.25 ms; 95 and 2.62 ms with scalar gathers and sums and the spline weights of
+// each position apart).  On the 268 M particle beam 30.0 ms against 34.2.
 #include "pp_sorted.cuh"
 #include "pp_tma.cuh"
 
@@ -70,7 +78,19 @@ constexpr int kWG = kT + kRLo + 2;                             // 12
 constexpr int kFComp = (kWG * kWG * kWG + 31) / 32 * 32;       // 1728 words
 constexpr uint32_t kFBoxBytes = sizeof(float) * kWG * kWG * kWG;  // 6912 bytes per component
 constexpr size_t kFieldBytes = sizeof(float) * 6 * kFComp + 128;
-__device__ __forceinline__ int fi(int i, int j, int k) { return i + kWG * (j + kWG * k); }
+// The gather reads the window as pairs: every node with its neighbour along x,
+// 12 pairs a row (the last one's neighbour is 0), so that a row of a support is
+// one or two aligned 8-byte shared loads from any start.  The lanes of a warp
+// sit in one or two cells: the loads are broadcasts, one wavefront each as a
+// 4-byte load's are.  Shared memory holds the pairs of two planes of cells (six
+// of nodes); the particles of a chunk, sorted by cell, pass through them in
+// turn.  A step along x, y and z is 2, 24 and 16 words modulo the 32 banks, so
+// that the up to eight starts that one cell's particles have (one per octant)
+// fall in distinct banks.
+constexpr int kPZ = 2;                                         // cell planes of the pairs
+constexpr int kPRow = kWG, kPPlane = kWG * kPRow + 8, kPComp = (kPZ + 4) * kPPlane;   // in pairs
+static_assert(kPRow * 2 % 32 == 24 && kPPlane * 2 % 32 == 16, "pair strides");
+constexpr size_t kPairBytes = 6 * kPComp * 8;
 // A staging wait that has not completed after this long gives up (ST_TIMEOUT).
 constexpr uint64_t kStageWaitNs = 1000000000ull;
 #ifndef PP_CELLS_CHUNK
@@ -105,7 +125,10 @@ constexpr int kMisc = 20 + 4 * kCPer * kCW;
 // A crossing piece is stored as its first queue entry (12 bits) and its
 // length - 1 (3 bits).
 static_assert(kCC <= 4096 && kPiece <= 8, "crossing-piece word");
-constexpr size_t kCellsSmem = kFieldBytes + sizeof(float) * (3 * kWVol + 6 * kCS) + sizeof(uint16_t) * (4 * kCC + 4) +
+// The lists of pieces are built when the chunk's gathers are done: they take
+// the place of the pairs.
+static_assert(sizeof(uint16_t) * (3 * kCC + 4) <= kPairBytes, "piece lists");
+constexpr size_t kCellsSmem = kFieldBytes + kPairBytes + sizeof(float) * (3 * kWVol + 6 * kCS) + sizeof(uint16_t) * kCC +
                               sizeof(int) * kMisc;
 // The current window: an int32 fixed-point window whose unit each chunk takes
 // from its particles' motion, flushed into the FP32 mesh per chunk; or, with
@@ -132,22 +155,24 @@ static_assert(kCellsSmem <= 227 * 1024, "tile CTA must fit the opt-in shared mem
 
 __device__ __forceinline__ int wi(int i, int j, int k) { return i + kW * (j + kW * k); }
 
-// Gather accessor over the staged E/B window (frame = the particle's cell).
-struct CellsFieldAcc {
-    const float *Fw;
-    int base;
-    PP_IF_CHECKED(int wx = 0, wy = 0, wz = 0; int *st = nullptr; mutable int bad = 0;)
-#ifdef PP_CHECKED
-    __device__ __forceinline__ bool inside(int i, int j, int k) const {
-        return wx + i >= 0 && wx + i < kWG && wy + j >= 0 && wy + j < kWG && wz + k >= 0 && wz + k < kWG;
+// Rows of the window's pairs, for the gather.
+struct PairRow {
+    const f2 *q;
+    template <bool both>
+    __device__ __forceinline__ ulonglong2 pairs(int j, int k) const {
+        const f2 *r = q + k * kPPlane + j * kPRow;
+        return make_ulonglong2(r[0], both ? r[2] : 0);
     }
-    __device__ ~CellsFieldAcc() {
-        if (bad && st) atomicOr(st, ST_BOUNDS);
-    }
-#endif
-    __device__ __forceinline__ float F(int kind, int comp, int i, int j, int k) const {
-        PP_IF_CHECKED(if (!inside(i, j, k)) { bad = 1; return 0.0f; })
-        return Fw[(kind * 3 + comp) * kFComp + base + fi(i, j, k)];
+};
+struct PairWindow {
+    const f2 *q;   // at the node two below the particle's cell
+    PP_IF_CHECKED(int rx, ry, rz, O; int *status;)
+    __device__ __forceinline__ PairRow operator()(int comp, int x, int y, int z) const {
+        PP_IF_CHECKED(if (rx + x + 2 * (O >= 2) >= kPRow || ry + y + O >= kWG || rz + z + O >= kPZ + 4) {
+            atomicOr(status, ST_BOUNDS);
+            return PairRow{q};
+        })
+        return PairRow{q + comp * kPComp + z * kPPlane + y * kPRow + x};
     }
 };
 
@@ -204,23 +229,55 @@ __device__ __forceinline__ void group_frame(int grp, int (&cw)[3], int (&lo)[3])
     }
 }
 
+// Old and new fractional coordinates along the axes, from the offset x0 and the
+// displacement d of a particle whose old support starts at the group's start
+// (coordinate 0 of the support: the cell for odd orders, the middle of the cell
+// or of the one below for even ones) and whose new one starts `step` nodes up.
+template <int O>
+__device__ __forceinline__ float group_origin(int grp, int axis) {
+    return O % 2 == 0 ? (((grp >> axis) & 1) ? 0.5f : -0.5f) : 0.0f;
+}
+
+// Prefix of dS along the current's axis on the lower faces, suffix on the upper
+// ones (they sum to zero), times the scale.
+template <int O, int NA, int N>
+__device__ __forceinline__ void face_prefix(const float (&DS)[N], float jscale, float (&C)[NA]) {
+    float run = 0.0f;
+#pragma unroll
+    for (int m = 0; m < NA; ++m) {
+        if (2 * m < O + 1) {
+            run += DS[m];
+            C[m] = run * jscale;
+        }
+    }
+    run = 0.0f;
+#pragma unroll
+    for (int m = NA - 1; m >= 0; --m) {
+        if (2 * m >= O + 1) {
+            run -= DS[m + 1];
+            C[m] = run * jscale;
+        }
+    }
+}
+
 // Component A of the current of the piece [s, e): the particles that cross no
 // support boundary (flag clear) share the support start lo, so their
 // O (O+1)^2 site values (those of deposit_esirkepov_inner, site by site) are
-// summed in registers and added once.
+// summed in registers, two nodes of axis B to a packed pair, and added once.
 template <int O, int A>
 __device__ __forceinline__ void piece_current(JT *Jw, const float *s_o, const float *s_d, const uint16_t *s_grp,
                                               int s, int e, float jscale PP_IF_CHECKED(, int *st)) {
-    constexpr int Bx = (A + 1) % 3, Cx = (A + 2) % 3;
+    constexpr int Bx = (A + 1) % 3, Cx = (A + 2) % 3, NP = (O + 2) / 2;
+    const int grp = s_grp[s] & kGrpMask;
     int cw[3], lo[3];
-    group_frame<O>(s_grp[s] & kGrpMask, cw, lo);
-    float acc[O][O + 1][O + 1];
+    group_frame<O>(grp, cw, lo);
+    f2 acc[O][NP][O + 1];
 #pragma unroll
     for (int m = 0; m < O; ++m)
 #pragma unroll
-        for (int mb = 0; mb <= O; ++mb)
+        for (int mb = 0; mb < NP; ++mb)
 #pragma unroll
-            for (int mc = 0; mc <= O; ++mc) acc[m][mb][mc] = 0.0f;
+            for (int mc = 0; mc <= O; ++mc) acc[m][mb][mc] = 0;
 #pragma unroll 1
     for (int q = s; q < e; ++q) {
         if (s_grp[q] & kSkip) continue;
@@ -228,43 +285,29 @@ __device__ __forceinline__ void piece_current(JT *Jw, const float *s_o, const fl
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             const float x0 = s_o[d * kCS + sp(q)];
-            const float x1 = x0 + s_d[d * kCS + sp(q)];
-            float wo[O + 1], wn[O + 1];
-            support<O, float>(x0, false, wo);
-            support<O, float>(x1, false, wn);
+            const float x1 = x0 + s_d[d * kCS + sp(q)], org = group_origin<O>(grp, d);
+            float wn[O + 1];
+            bspline2<O>(x0 - org, x1 - org, S0[d], wn);
 #pragma unroll
-            for (int m = 0; m <= O; ++m) {
-                S0[d][m] = wo[m];
-                DS[d][m] = wn[m] - wo[m];
-            }
+            for (int m = 0; m <= O; ++m) DS[d][m] = wn[m] - S0[d][m];
         }
-        // prefix of dS along A (suffix form on the upper faces; the last face is 0)
         float C[O];
-        float run = 0.0f;
+        face_prefix<O, O>(DS[A], jscale, C);
+        f2 sb[NP], db[NP];
 #pragma unroll
-        for (int m = 0; m < O; ++m) {
-            if (2 * m < O + 1) {
-                run += DS[A][m];
-                C[m] = run * jscale;
-            }
-        }
-        run = 0.0f;
-#pragma unroll
-        for (int m = O - 1; m >= 0; --m) {
-            if (2 * m >= O + 1) {
-                run -= DS[A][m + 1];
-                C[m] = run * jscale;
-            }
+        for (int mb = 0; mb < NP; ++mb) {
+            sb[mb] = pack2(S0[Bx][2 * mb], 2 * mb < O ? S0[Bx][2 * mb + 1] : 0.0f);
+            db[mb] = pack2(DS[Bx][2 * mb], 2 * mb < O ? DS[Bx][2 * mb + 1] : 0.0f);
         }
 #pragma unroll
         for (int mc = 0; mc <= O; ++mc) {
-            const float p = S0[Cx][mc] + 0.5f * DS[Cx][mc];
-            const float h = 0.5f * S0[Cx][mc] + (1.0f / 3.0f) * DS[Cx][mc];
+            const f2 p = dup2(S0[Cx][mc] + 0.5f * DS[Cx][mc]);
+            const f2 h = dup2(0.5f * S0[Cx][mc] + (1.0f / 3.0f) * DS[Cx][mc]);
 #pragma unroll
-            for (int mb = 0; mb <= O; ++mb) {
-                const float Y = S0[Bx][mb] * p + DS[Bx][mb] * h;
+            for (int mb = 0; mb < NP; ++mb) {
+                const f2 Y = fma2(sb[mb], p, mul2(db[mb], h));
 #pragma unroll
-                for (int m = 0; m < O; ++m) acc[m][mb][mc] += C[m] * Y;
+                for (int m = 0; m < O; ++m) acc[m][mb][mc] = fma2(dup2(C[m]), Y, acc[m][mb][mc]);
             }
         }
     }
@@ -284,7 +327,9 @@ __device__ __forceinline__ void piece_current(JT *Jw, const float *s_o, const fl
                     continue;
                 }
 #endif
-                jadd(Jw + A * kWVol + wi(idx[0], idx[1], idx[2]), acc[m][mb][mc]);
+                float v[2];
+                unpack2(acc[m][mb / 2][mc], v[0], v[1]);
+                jadd(Jw + A * kWVol + wi(idx[0], idx[1], idx[2]), v[mb % 2]);
             }
 }
 
@@ -330,25 +375,30 @@ __device__ __forceinline__ void cross_piece(JT *Jw, int A, int XA, const float *
                                             float jscale PP_IF_CHECKED(, int *st)) {
     constexpr int RB = (RA + 1) % 3, RC = (RA + 2) % 3;
     constexpr int NA = (RA == 0) ? O + 1 : O;
-    constexpr int NB = (RB == 0) ? O + 2 : O + 1;
-    constexpr int NC = (RC == 0) ? O + 2 : O + 1;
+    // pairs run along an axis that is not the crossing one: B, or C where B is
+    constexpr bool kPairC = RB == 0;
+    constexpr int RP = kPairC ? RC : RB, RS = kPairC ? RB : RC;   // axes of the pairs and of the single nodes
+    constexpr int NP = (O + 2) / 2, NS = (RS == 0) ? O + 2 : O + 1;
     int cw[3], lo[3];
     group_frame<O>(grp, cw, lo);
     const int p[3] = {XA, XA == 2 ? 0 : XA + 1, XA == 0 ? 2 : XA - 1};   // physical axis of rotated axis r
     int lr[3], sr[3];   // support start and window stride per rotated axis
+    float org[3];
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
         lr[r] = p[r] == 0 ? lo[0] : (p[r] == 1 ? lo[1] : lo[2]);
         sr[r] = p[r] == 0 ? 1 : (p[r] == 1 ? kW : kW * kW);
+        org[r] = group_origin<O>(grp, p[r]);
     }
     lr[0] -= up ? 0 : 1;   // union start along the crossing axis: the lower of the old and new starts
-    float acc[NA][NB][NC];
+    const float step = up ? 1.0f : -1.0f;
+    f2 acc[NA][NP][NS];
 #pragma unroll
     for (int m = 0; m < NA; ++m)
 #pragma unroll
-        for (int mb = 0; mb < NB; ++mb)
+        for (int mp = 0; mp < NP; ++mp)
 #pragma unroll
-            for (int mc = 0; mc < NC; ++mc) acc[m][mb][mc] = 0.0f;
+            for (int ms = 0; ms < NS; ++ms) acc[m][mp][ms] = 0;
 #pragma unroll 1
     for (int e = ks; e < ke; ++e) {
         const int q = s_queue[e];
@@ -358,8 +408,7 @@ __device__ __forceinline__ void cross_piece(JT *Jw, int A, int XA, const float *
             const float x0 = s_o[p[r] * kCS + sp(q)];
             const float x1 = x0 + s_d[p[r] * kCS + sp(q)];
             float wo[O + 1], wn[O + 1];
-            support<O, float>(x0, false, wo);
-            support<O, float>(x1, false, wn);
+            bspline2<O>(x0 - org[r], r == 0 ? x1 - org[r] - step : x1 - org[r], wo, wn);
             if (r == 0) {   // old weights from the union start (up) or one node above it
 #pragma unroll
                 for (int m = 0; m < O + 2; ++m) {
@@ -378,33 +427,23 @@ __device__ __forceinline__ void cross_piece(JT *Jw, int A, int XA, const float *
                 DS[r][O + 1] = 0.0f;
             }
         }
-        // prefix of dS along A on the lower faces, suffix on the upper ones
         float C[NA];
-        float run = 0.0f;
+        face_prefix<O, NA>(DS[RA], jscale, C);
+        f2 sb[NP], db[NP];
 #pragma unroll
-        for (int m = 0; m < NA; ++m) {
-            if (2 * m < O + 1) {
-                run += DS[RA][m];
-                C[m] = run * jscale;
-            }
-        }
-        run = 0.0f;
-#pragma unroll
-        for (int m = NA - 1; m >= 0; --m) {
-            if (2 * m >= O + 1) {
-                run -= DS[RA][m + 1];
-                C[m] = run * jscale;
-            }
+        for (int mp = 0; mp < NP; ++mp) {
+            sb[mp] = pack2(S0[RP][2 * mp], S0[RP][2 * mp + 1]);
+            db[mp] = pack2(DS[RP][2 * mp], DS[RP][2 * mp + 1]);
         }
 #pragma unroll
-        for (int mc = 0; mc < NC; ++mc) {
-            const float pc = S0[RC][mc] + 0.5f * DS[RC][mc];
-            const float hc = 0.5f * S0[RC][mc] + (1.0f / 3.0f) * DS[RC][mc];
+        for (int ms = 0; ms < NS; ++ms) {
+            const f2 pc = dup2(S0[RS][ms] + 0.5f * DS[RS][ms]);
+            const f2 hc = dup2(0.5f * S0[RS][ms] + (1.0f / 3.0f) * DS[RS][ms]);
 #pragma unroll
-            for (int mb = 0; mb < NB; ++mb) {
-                const float Y = S0[RB][mb] * pc + DS[RB][mb] * hc;
+            for (int mp = 0; mp < NP; ++mp) {
+                const f2 Y = fma2(sb[mp], pc, mul2(db[mp], hc));
 #pragma unroll
-                for (int m = 0; m < NA; ++m) acc[m][mb][mc] += C[m] * Y;
+                for (int m = 0; m < NA; ++m) acc[m][mp][ms] = fma2(dup2(C[m]), Y, acc[m][mp][ms]);
             }
         }
     }
@@ -412,17 +451,19 @@ __device__ __forceinline__ void cross_piece(JT *Jw, int A, int XA, const float *
 #pragma unroll
     for (int m = 0; m < NA; ++m)
 #pragma unroll
-        for (int mb = 0; mb < NB; ++mb)
+        for (int mp = 0; mp <= O; ++mp)
 #pragma unroll
-            for (int mc = 0; mc < NC; ++mc) {
+            for (int ms = 0; ms < NS; ++ms) {
 #ifdef PP_CHECKED
-                if (lr[RA] + m < 0 || lr[RA] + m >= kW || lr[RB] + mb < 0 || lr[RB] + mb >= kW || lr[RC] + mc < 0 ||
-                    lr[RC] + mc >= kW) {
+                if (lr[RA] + m < 0 || lr[RA] + m >= kW || lr[RP] + mp < 0 || lr[RP] + mp >= kW || lr[RS] + ms < 0 ||
+                    lr[RS] + ms >= kW) {
                     atomicOr(st, ST_BOUNDS);
                     continue;
                 }
 #endif
-                jadd(J + (lr[RA] + m) * sr[RA] + (lr[RB] + mb) * sr[RB] + (lr[RC] + mc) * sr[RC], acc[m][mb][mc]);
+                float v[2];
+                unpack2(acc[m][mp / 2][ms], v[0], v[1]);
+                jadd(J + (lr[RA] + m) * sr[RA] + (lr[RP] + mp) * sr[RP] + (lr[RS] + ms) * sr[RS], v[mp % 2]);
             }
 }
 
@@ -493,14 +534,15 @@ template <int O, int PUSH, bool BND, bool GMAPS>
 __device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int tile, float *smem, uint32_t &phase) {
     float *F = smem;
     uint64_t *bar = (uint64_t *)((char *)smem + kFieldBytes - 128);
-    JT *Jw = (JT *)((char *)smem + kFieldBytes);
+    f2 *Fp = (f2 *)((char *)smem + kFieldBytes);       // pairs of the gather, then the lists of pieces
+    JT *Jw = (JT *)((char *)smem + kFieldBytes + kPairBytes);
     float *s_o = (float *)(Jw + 3 * kWVol);   // 3 x kCS: offsets at t (frame of the cell)
     float *s_d = s_o + 3 * kCS;           // 3 x kCS: displacement of the step
     uint16_t *s_grp = (uint16_t *)(s_d + 3 * kCS);   // group word (deposit group, crossing, kSkip)
-    uint16_t *s_piece = s_grp + kCC;                  // piece starts (+ the end)
+    uint16_t *s_piece = (uint16_t *)Fp;               // piece starts (+ the end)
     uint16_t *s_queue = s_piece + kCC + 2;            // crossing particles, in chunk order
     uint16_t *s_xpiece = s_queue + kCC;               // crossing pieces by bucket: first entry | (length - 1) << 12
-    int *misc = (int *)(s_xpiece + kCC + 2);   // [0]: queue length; [2]: pieces;
+    int *misc = (int *)(s_grp + kCC);   // [0]: queue length; [2]: pieces;
                                                // [4..9]: fixed point: cell box of the chunk; [10..12]: sum |dxi|
     int *cnt = misc + 16;                 // starts per (round, warp); four tables
     int *qcnt = cnt + kCPer * kCW;        // crossing particles per (round, warp)
@@ -547,7 +589,10 @@ __device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int tile, f
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int s = 0; s < T.ns; ++s) {
         const CellsSpecies &S = T.sp[s];
-        const int tb = S.cell_start[key0], te = S.cell_start[key1];
+        int sb[kT / kPZ + 1];   // the slabs' first particles
+#pragma unroll
+        for (int m = 0; m <= kT / kPZ; ++m) sb[m] = S.cell_start[key0 + m * kPZ * kT * kT * kSubKeys];
+        const int tb = sb[0], te = sb[kT / kPZ];
         for (int cb = tb; cb < te; cb += kCC) {
             const int cn = min(kCC, te - cb);
 #if PP_CELLS_FIXED
@@ -560,93 +605,121 @@ __device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int tile, f
             // dependent global loads overlap the gather
             int32_t n_cw = 0;
             float n_o[3] = {0.0f, 0.0f, 0.0f}, n_u[3] = {0.0f, 0.0f, 0.0f};
-            auto fetch = [&](int qf) {
-                if (qf >= cn) return;
+            auto fetch = [&](int qf, int end) {
+                if (qf >= end) return;
                 const int64_t i = (int64_t)cb + qf;
                 const int64_t src = S.perm ? (int64_t)S.perm[i] : i;
                 n_cw = S.p.cell[src];
                 n_o[0] = S.p.ox[src]; n_o[1] = S.p.oy[src]; n_o[2] = S.p.oz[src];
                 n_u[0] = S.p.ux[src]; n_u[1] = S.p.uy[src]; n_u[2] = S.p.uz[src];
             };
-            fetch(threadIdx.x);
 #pragma unroll 1
-            for (int r = 0; r < kCPer; ++r) {
-                const int q = r * kCT + threadIdx.x;
-                if (q >= cn) break;
-                const int64_t idx = (int64_t)cb + q;
-                const int32_t cw0 = n_cw;
-                float xi0[3] = {n_o[0], n_o[1], n_o[2]};
-                float u[3] = {n_u[0], n_u[1], n_u[2]};
-                fetch(q + kCT);
-                int cx, cy, cz;
-                unpack_cell(cw0, cx, cy, cz);
-                const int rx = cx - ox, ry = cy - oy, rz = cz - oz;
-                if ((unsigned)rx >= (unsigned)kT || (unsigned)ry >= (unsigned)kT || (unsigned)rz >= (unsigned)kT) {
-                    // not in its sorted tile: cannot happen after a sort; left unmoved and flagged
-                    atomicOr(T.status, ST_RANGE);
-                    s_grp[q] = kSkip;
-                    store_sorted(T, S, idx, cw0, xi0, u);
-                    continue;
-                }
-                const float u0[3] = {u[0], u[1], u[2]};
-                const int grp = group_of<O>(rx, ry, rz, xi0);
-                if (S.qmdt != 0.0f) {   // uniform: no kick, no force
-                    float E[3], B[3];
-                    CellsFieldAcc facc{F, fi(rx + kRLo, ry + kRLo, rz + kRLo)};
-                    PP_IF_CHECKED(facc.wx = rx + kRLo; facc.wy = ry + kRLo; facc.wz = rz + kRLo; facc.st = T.status;)
-                    gather_EB<O, float>(facc, xi0, E, B);
-                    push_particle<PUSH, float>(S.qmdt, S.kdt, E, B, u);
-                }
-                const float gi = 1.0f / sqrtf(1.0f + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-                float dx[3], xi1[3];
-                bool ok = true;
-                int ncross = 0, xa = 0;
+            for (int slab = 0; slab < kT / kPZ; ++slab) {
+                int s0 = sb[0], s1 = sb[1];   // sb[slab], sb[slab + 1] without a run-time index
 #pragma unroll
-                for (int d = 0; d < 3; ++d) {
-                    dx[d] = T.dtdx[d] * u[d] * gi;
-                    xi1[d] = xi0[d] + dx[d];
-                    ok = ok && (fabsf(dx[d]) < 1.0f);
-                    if (floorf(xi0[d] - 0.5f * (O - 1)) != floorf(xi1[d] - 0.5f * (O - 1))) {
-                        ++ncross;
-                        xa = d;
+                for (int m = 1; m < kT / kPZ; ++m)
+                    if (slab == m) {
+                        s0 = sb[m];
+                        s1 = sb[m + 1];
                     }
+                const int qa = max(cb, s0) - cb, qe = min(cb + cn, s1) - cb;
+                if (qa >= qe) continue;
+                fetch(qa + threadIdx.x, qe);
+                __syncthreads();   // the last slab's gathers, or the last chunk's pieces, are done
+                for (int t = threadIdx.x; t < 6 * (kPZ + 4) * kWG; t += kCT) {   // window rows to pairs
+                    const int c = t / ((kPZ + 4) * kWG), r = t - c * (kPZ + 4) * kWG;
+                    const float4 *src = reinterpret_cast<const float4 *>(F + c * kFComp + (slab * kPZ * kWG + r) * kWG);
+                    float4 *dst = reinterpret_cast<float4 *>(Fp + c * kPComp + (r / kWG) * kPPlane + (r % kWG) * kPRow);
+                    const float4 a = src[0], b = src[1], d = src[2];
+                    dst[0] = make_float4(a.x, a.y, a.y, a.z);
+                    dst[1] = make_float4(a.z, a.w, a.w, b.x);
+                    dst[2] = make_float4(b.x, b.y, b.y, b.z);
+                    dst[3] = make_float4(b.z, b.w, b.w, d.x);
+                    dst[4] = make_float4(d.x, d.y, d.y, d.z);
+                    dst[5] = make_float4(d.z, d.w, d.w, 0.0f);
                 }
-                if (!ok) {   // leave the particle unchanged and flag the step
-                    atomicOr(T.status, isfinite(u[0] + u[1] + u[2]) ? ST_CFL : ST_NAN);
-                    s_grp[q] = (uint16_t)(grp | kSkip);
-                    store_sorted(T, S, idx, cw0, xi0, u0);
-                    continue;
-                }
+                __syncthreads();
+#pragma unroll 1
+                for (int q = qa + threadIdx.x; q < qe; q += kCT) {
+                    const int64_t idx = (int64_t)cb + q;
+                    const int32_t cw0 = n_cw;
+                    const float xi0[3] = {n_o[0], n_o[1], n_o[2]};
+                    float u[3] = {n_u[0], n_u[1], n_u[2]};
+                    fetch(q + kCT, qe);
+                    int cc[3];
+                    unpack_cell(cw0, cc[0], cc[1], cc[2]);
+                    int rx = cc[0] - ox, ry = cc[1] - oy, rz = cc[2] - oz - slab * kPZ;
+                    const bool here = (unsigned)rx < (unsigned)kT && (unsigned)ry < (unsigned)kT && (unsigned)rz < (unsigned)kPZ;
+                    if (!here) rx = ry = rz = 0;
+                    const float u0[3] = {u[0], u[1], u[2]};
+                    const int grp = group_of<O>(rx, ry, rz + slab * kPZ, xi0);
+                    if (S.qmdt != 0.0f) {   // uniform: no kick, no force
+                        float E[3] = {0.0f, 0.0f, 0.0f}, B[3] = {0.0f, 0.0f, 0.0f};
+                        gather_pairs<O>(PairWindow{Fp + rz * kPPlane + ry * kPRow + rx PP_IF_CHECKED(, rx, ry, rz, O, T.status)},
+                                        xi0, E, B);
+                        push_particle<PUSH, float>(S.qmdt, S.kdt, E, B, u);
+                    }
+                    const float gi = inv_sqrt(1.0f + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+                    float dx[3], xi1[3];
+                    bool ok = here;
+                    int ncross = 0, xa = 0;
 #pragma unroll
-                for (int d = 0; d < 3; ++d) {
-                    s_o[d * kCS + sp(q)] = xi0[d];
-                    s_d[d * kCS + sp(q)] = dx[d];
-                }
+                    for (int d = 0; d < 3; ++d) {
+                        dx[d] = T.dtdx[d] * u[d] * gi;
+                        xi1[d] = xi0[d] + dx[d];
+                        ok = ok && (fabsf(dx[d]) < 1.0f);
+                        if (floorf(xi0[d] - 0.5f * (O - 1)) != floorf(xi1[d] - 0.5f * (O - 1))) {
+                            ++ncross;
+                            xa = d;
+                        }
+                    }
+                    if (!ok) {
+                        // not in its sorted place (cannot happen after a sort), a cell or more in one
+                        // step, or not finite: left unchanged, and the step flagged
+                        atomicOr(T.status, !here ? ST_RANGE : (isfinite(u[0] + u[1] + u[2]) ? ST_CFL : ST_NAN));
+                        s_grp[q] = (uint16_t)(grp | kSkip);
+                        store_sorted(T, S, idx, cw0, xi0, u0);
+                        continue;
+                    }
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        s_o[d * kCS + sp(q)] = xi0[d];
+                        s_d[d * kCS + sp(q)] = dx[d];
+                    }
 #if PP_CELLS_FIXED
-                sum[0] += fabsf(dx[0]); sum[1] += fabsf(dx[1]); sum[2] += fabsf(dx[2]);
-                blo[0] = min(blo[0], rx); blo[1] = min(blo[1], ry); blo[2] = min(blo[2], rz);
-                bhi[0] = max(bhi[0], rx); bhi[1] = max(bhi[1], ry); bhi[2] = max(bhi[2], rz);
+                    sum[0] += fabsf(dx[0]); sum[1] += fabsf(dx[1]); sum[2] += fabsf(dx[2]);
+                    blo[0] = min(blo[0], rx); blo[1] = min(blo[1], ry); blo[2] = min(blo[2], rz + slab * kPZ);
+                    bhi[0] = max(bhi[0], rx); bhi[1] = max(bhi[1], ry); bhi[2] = max(bhi[2], rz + slab * kPZ);
 #endif
-                // crossing signature: the axis and direction of a support start
-                // that moves on one axis alone, 7 when it moves on several
-                const int sig = ncross == 0 ? 0 : (ncross == 1 ? 1 + 2 * xa + (dx[xa] > 0.0f ? 1 : 0) : 7);
-                s_grp[q] = (uint16_t)(grp | (sig << kSigShift) | (ncross ? kSkip : 0));
-                // the new state, written to the slot (the deposit reads the staged copy)
-                int ncx = cx, ncy = cy, ncz = cz;
-                rebin(xi1[0], ncx, g.n[0]);
-                rebin(xi1[1], ncy, g.n[1]);
-                rebin(xi1[2], ncz, g.n[2]);
-                int32_t cwd;
-                if constexpr (BND) {
-                    reflect(ncx, xi1[0], u[0], T.wall[0]);
-                    reflect(ncy, xi1[1], u[1], T.wall[1]);
-                    reflect(ncz, xi1[2], u[2], T.wall[2]);
-                    cwd = pack_cell(ncx, ncy, ncz);
-                    if (T.esc > 0.0 && (double)ncx + (double)xi1[0] < T.esc && u[0] < 0.0f) cwd |= kDeadBit;
-                } else {
-                    cwd = pack_cell(ncx, ncy, ncz);
+                    // crossing signature: the axis and direction of a support start
+                    // that moves on one axis alone, 7 when it moves on several
+                    const float dxa = xa == 0 ? dx[0] : (xa == 1 ? dx[1] : dx[2]);
+                    const int sig = ncross == 0 ? 0 : (ncross == 1 ? 1 + 2 * xa + (dxa > 0.0f ? 1 : 0) : 7);
+                    s_grp[q] = (uint16_t)(grp | (sig << kSigShift) | (ncross ? kSkip : 0));
+                    // the new state, written to the slot (the deposit reads the staged copy): the
+                    // offset back into [0, 1), the cell wrapped
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        const float fl = floorf(xi1[d]);
+                        xi1[d] -= fl;
+                        int c = cc[d] + (int)fl;
+                        if (xi1[d] >= 1.0f) {   // a small negative offset that rounds to 1
+                            xi1[d] = 0.0f;
+                            ++c;
+                        }
+                        c = c < 0 ? c + g.n[d] : c;
+                        cc[d] = c >= g.n[d] ? c - g.n[d] : c;
+                    }
+                    int32_t cwd = pack_cell(cc[0], cc[1], cc[2]);
+                    if constexpr (BND) {
+                        reflect(cc[0], xi1[0], u[0], T.wall[0]);
+                        reflect(cc[1], xi1[1], u[1], T.wall[1]);
+                        reflect(cc[2], xi1[2], u[2], T.wall[2]);
+                        cwd = pack_cell(cc[0], cc[1], cc[2]);
+                        if (T.esc > 0.0 && (double)cc[0] + (double)xi1[0] < T.esc && u[0] < 0.0f) cwd |= kDeadBit;
+                    }
+                    store_sorted(T, S, idx, cwd, xi1, u);
                 }
-                store_sorted(T, S, idx, cwd, xi1, u);
             }
 #if PP_CELLS_FIXED
             if (threadIdx.x < 3) {   // previous chunk's values were last read before the barrier above

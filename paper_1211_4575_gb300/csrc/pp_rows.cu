@@ -121,29 +121,6 @@ struct AxisMove {
 };
 constexpr float kRsqrt12 = 0.28867513459481287f;
 
-// bspline of two fractional coordinates at once, packed.
-template <int O>
-__device__ __forceinline__ void bspline2(float fa, float fb, float (&a)[O + 1], float (&b)[O + 1]) {
-    const f2 f = pack2(fa, fb), one = dup2(1.0f);
-    const f2 g = fma2(f, dup2(-1.0f), one);
-    if constexpr (O == 1) {
-        unpack2(g, a[0], b[0]);
-        unpack2(f, a[1], b[1]);
-    } else if constexpr (O == 2) {
-        const f2 h = fma2(one, f, dup2(-0.5f));
-        unpack2(mul2(mul2(g, g), dup2(0.5f)), a[0], b[0]);
-        unpack2(fma2(mul2(h, dup2(-1.0f)), h, dup2(0.75f)), a[1], b[1]);
-        unpack2(mul2(mul2(f, f), dup2(0.5f)), a[2], b[2]);
-    } else {
-        // w1 = (3 f^3 - 6 f^2 + 4) / 6 = 2/3 - f^2 (1 - f/2), and w2 the same in g = 1 - f
-        const f2 ff = mul2(f, f), gg = mul2(g, g), m = dup2(0.5f), c = dup2(2.0f / 3.0f), s = dup2(1.0f / 6.0f);
-        unpack2(mul2(mul2(gg, s), g), a[0], b[0]);
-        unpack2(fma2(ff, fma2(f, m, dup2(-1.0f)), c), a[1], b[1]);
-        unpack2(fma2(gg, fma2(g, m, dup2(-1.0f)), c), a[2], b[2]);
-        unpack2(mul2(mul2(ff, s), f), a[3], b[3]);
-    }
-}
-
 template <int O>
 __device__ __forceinline__ void axis_move(float o, float d, float js, AxisMove &r) {
     float w0[O + 1], w[O + 1], f0, f1, S0[4], S1[4];
