@@ -631,10 +631,12 @@ __global__ void __launch_bounds__(256) k_rhs_lin(Geom g, const __grid_constant__
 // One Chebyshev sweep (Saad's three-term form, see field_update_impl):
 // r = rhs - X + kk L X, X_new = X + c1 (X - X_prev) + c2 r.  A thread marches
 // through zper planes of one component with the 11 nodes along z in registers.
-// FP32 on large meshes: bound by the L1 and L2 traffic of the neighbours;
-// FP64: by the part's FP64 rate (about 40 operations a node and component);
-// small meshes: by launch and load latency, so the march is cut until every
-// SM has threads.  CHEB_FIG
+// FP32 on large meshes: bound by the latency of the neighbours' loads (L1 and
+// L2), so a plane's streams are loaded one plane ahead; FP64: by the part's FP64
+// rate (about 40 operations a node and component); small meshes: by launch and
+// load latency, so the march is cut until every SM has threads.  Blocks of 32 x
+// 16 nodes and six planes (256 x 128 x 128 nodes, the whole field update: 1.66 ms;
+// 64 x 8 nodes 1.68; 16 planes 1.80; without the loads ahead 2.16).
 template <typename R, int W>
 __global__ void __launch_bounds__(256) k_cheb(Geom g, const __grid_constant__ Coef<R> k, Vec3<R> X, Vec3<R> Xp,
                                               Vec3<R> Rh, R *O0, R *O1, R *O2, R kk, R c1, R c2, int zper, int nzc) {
@@ -648,8 +650,16 @@ __global__ void __launch_bounds__(256) k_cheb(Geom g, const __grid_constant__ Co
     Nodes<R, W> col[11];
 #pragma unroll
     for (int m = 0; m < 11; ++m) col[m] = ld<W>(f + q + (m - 5) * sz);
+    // the previous iterate and rhs one plane ahead, the column's top two
+    Nodes<R, W> xpn = ld<W>(fp + q), rzn = ld<W>(rh + q), top = col[10];
+    if (z0 + 1 < z1) top = ld<W>(f + q + 6 * sz);
     for (int z = z0;;) {
-        const Nodes<R, W> xp = ld<W>(fp + q), rz = ld<W>(rh + q);
+        const Nodes<R, W> xp = xpn, rz = rzn, next = top;
+        if (z + 1 < z1) {
+            xpn = ld<W>(fp + q + sz);
+            rzn = ld<W>(rh + q + sz);
+            if (z + 2 < z1) top = ld<W>(f + q + 7 * sz);
+        }
         const Nodes<R, W> L = laplace<R, W>(f + q, sy, col, k);
         Nodes<R, W> nv;
 #pragma unroll
@@ -663,7 +673,7 @@ __global__ void __launch_bounds__(256) k_cheb(Geom g, const __grid_constant__ Co
         q += sz;
 #pragma unroll
         for (int m = 0; m < 10; ++m) col[m] = col[m + 1];
-        col[10] = ld<W>(f + q + 5 * sz);
+        col[10] = next;
     }
 }
 
@@ -765,8 +775,9 @@ static Coef<R> coef_of(const FieldCoef &k) {
     return r;
 }
 
-// Planes a thread marches through: as many as leave kMarchBlocks blocks.  A
-// march of zper planes reads zper + 10 of them.
+// Planes a thread marches through: six, or as many as leave kMarchBlocks blocks
+// (six per SM; 64^3 nodes: 0.216 ms with one plane, 0.232 with two, 0.277 with
+// six; 128 x 64 x 64: 0.330 with two or three, 0.341 with one, 0.360 with six).
 constexpr int kMarchBlocks = 912;
 
 template <typename R, int W>
@@ -779,10 +790,10 @@ static cudaError_t field_update_impl(Ctx &c) {
     const Ctx::Cheb &ch = c.cheb[c.cheb_sel];
     cudaError_t e;
     // blocks of 256 threads (64 for FP64, whose rate wants every SM busy), as wide
-    // along x as the rows need
+    // along x as the rows need, up to 16 threads
     const int nx = (g.n[0] + W - 1) / W, threads = sizeof(R) == 8 ? 64 : 256;
     int bx = 8;
-    while (bx < 32 && bx < nx) bx *= 2;
+    while (bx < 16 && bx < nx) bx *= 2;
     const dim3 blk((unsigned)bx, (unsigned)(threads / bx));
     dim3 grid((unsigned)((nx + bx - 1) / bx), (unsigned)((g.n[1] + blk.y - 1) / blk.y), (unsigned)(3 * g.n[2]));
     k_rhs_lin<R, W><<<grid, blk, 0, c.st>>>(g, k, v3<R>(c.E), v3<R>(c.B), v3<R>(c.J), (R *)c.R[0], (R *)c.R[1],
@@ -792,8 +803,8 @@ static cudaError_t field_update_impl(Ctx &c) {
     // Chebyshev semi-iteration on the spectrum [1, lmax] of the SPD operator,
     // starting from B^n (Saad, Iterative Methods, Alg. 12.1 in 3-term form).
     double theta = ch.theta, delta = ch.delta;
-    int zper = 16;
-    while (zper > 1 && (int64_t)grid.x * grid.y * 3 * ((g.n[2] + zper - 1) / zper) < kMarchBlocks) zper /= 2;
+    int zper = 6;
+    while (zper > 1 && (int64_t)grid.x * grid.y * 3 * ((g.n[2] + zper - 1) / zper) < kMarchBlocks) --zper;
     const int nzc = (g.n[2] + zper - 1) / zper;
     const dim3 pg(grid.x, grid.y, (unsigned)(3 * nzc));
     void **cur = c.B, **prev = c.B;
