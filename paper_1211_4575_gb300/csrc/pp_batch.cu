@@ -224,14 +224,14 @@ static bool fused_round(pp_batch *b) {
     for (int grp = 0; grp < pp_batch::kGroups; ++grp) {
         Ctx *g[4096];
         int m = 0;
-        int64_t tiles = 0;
+        int64_t items = 0;
         for (int k = 0; k < n; ++k)
             if (ok[k] && cells_batch_key(*run[k]) == grp) {
                 g[m++] = run[k];
-                tiles += (int64_t)run[k]->ntile[0] * run[k]->ntile[1] * run[k]->ntile[2];
+                items += cells_items(*run[k]);
             }
         if (m == 0) continue;
-        cudaError_t e = ensure_room(b, par, grp, cells_args_bytes() * m, sizeof(int2) * tiles);
+        cudaError_t e = ensure_room(b, par, grp, cells_args_bytes() * m, sizeof(int2) * items);
         // the pinned buffers of this parity were last read by the copies of two rounds ago
         if (e == cudaSuccess) e = cudaEventSynchronize(b->h_done[par][grp]);
         if (e == cudaSuccess)

@@ -524,14 +524,16 @@ __device__ __forceinline__ void scan_counts(int *c, int *total, int lane) {
 
 // BND: walls (reflection) and the open end (escape); a separate instantiation
 // so that periodic runs carry none of their tests.
-// One tile of one run: the whole particle step of the tile's particles (all
-// species), its current added into the run's mesh.  Called by every thread
-// of the CTA; smem is the CTA's dynamic shared memory.
+// One tile of one run: the whole particle step of the tile's particles of one
+// species (item: tile times species, plus the species), its current added into
+// the run's mesh.  Called by every thread of the CTA; smem is the CTA's dynamic
+// shared memory.  The chunks of the species are independent, so a species to a
+// CTA changes no sum but makes twice the blocks of a two-species plasma: SPLIT_FIG
 // Returns false when the CTA must stop: a staging wait ran out (here or in
 // another CTA, ST_TIMEOUT).  phase: parity of the CTA's staging mbarrier, which
 // the kernel initialised.  GMAPS: the tensor maps sit in global memory.
 template <int O, int PUSH, bool BND, bool GMAPS>
-__device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int tile, float *smem, uint32_t &phase) {
+__device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int item, float *smem, uint32_t &phase) {
     float *F = smem;
     uint64_t *bar = (uint64_t *)((char *)smem + kFieldBytes - 128);
     f2 *Fp = (f2 *)((char *)smem + kFieldBytes);       // pairs of the gather, then the lists of pieces
@@ -548,15 +550,14 @@ __device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int tile, f
     int *qcnt = cnt + kCPer * kCW;        // crossing particles per (round, warp)
     int *xtot = cnt + 4 * kCPer * kCW;    // crossing pieces per bucket
     const Geom &g = T.g;
+    const int tile = item / T.ns, s = item - tile * T.ns;
+    const CellsSpecies &S = T.sp[s];
     const int tx = tile % T.nt[0], ty = (tile / T.nt[0]) % T.nt[1], tz = tile / (T.nt[0] * T.nt[1]);
     const int ox = tx * kT, oy = ty * kT, oz = tz * kT;
     const int wx = ox - kRLo, wy = oy - kRLo, wz = oz - kRLo;
     const int64_t key0 = (int64_t)tile * kTCells * kSubKeys, key1 = key0 + kTCells * kSubKeys;
-    {   // a tile that holds no particle (the mirror half of a box between walls) stages nothing
-        int held = 0;
-        for (int s = 0; s < T.ns; ++s) held |= T.sp[s].cell_start[key1] - T.sp[s].cell_start[key0];
-        if (!held) return true;
-    }
+    // a tile that holds no particle (the mirror half of a box between walls) stages nothing
+    if (S.cell_start[key1] == S.cell_start[key0]) return true;
     // ---- the E/B window by six TMA tensor copies (array coordinates of the
     // window's first node; the host checked that every tile's box lies inside
     // the padded arrays with an aligned x; rechecked here, uniformly, so that
@@ -587,8 +588,7 @@ __device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int tile, f
     if (misc[3]) return false;
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int s = 0; s < T.ns; ++s) {
-        const CellsSpecies &S = T.sp[s];
+    {
         int sb[kT / kPZ + 1];   // the slabs' first particles
 #pragma unroll
         for (int m = 0; m <= kT / kPZ; ++m) sb[m] = S.cell_start[key0 + m * kPZ * kT * kT * kSubKeys];
@@ -935,7 +935,7 @@ __global__ void __launch_bounds__(kCT, 1) k_particles_cells(const __grid_constan
     cells_tile<O, PUSH, BND, false>(T, blockIdx.x, smem, phase);
 }
 
-// Batched form: the tiles of many runs as (run, tile) work items, taken in
+// Batched form: the tiles and species of many runs as (run, item) work items, taken in
 // order by persistent CTAs from a device counter (the items come sorted by
 // run size, largest first, so that the last items are short).  Every run's
 // arguments, tensor maps included, sit in device memory.
@@ -1002,7 +1002,7 @@ cudaError_t launch_particles_cells(Ctx &c) {
     bool any = false;
     cudaError_t ea = cells_args(c, T, any);
     if (ea != cudaSuccess || !any) return ea;
-    const unsigned blocks = (unsigned)(c.ntile[0] * c.ntile[1] * c.ntile[2]);
+    const unsigned blocks = (unsigned)((int64_t)c.ntile[0] * c.ntile[1] * c.ntile[2] * T.ns);
     const int o = c.d.shape_order, pu = c.d.pusher;
     const bool bnd = c.any_wall();
     static unsigned long long attr_done[2][2][4] = {};
@@ -1030,13 +1030,16 @@ cudaError_t launch_particles_cells(Ctx &c) {
     return cudaSuccess;
 }
 
+// Most work items of a context: its tiles times its species.
+int64_t cells_items(const Ctx &c) { return (int64_t)c.ntile[0] * c.ntile[1] * c.ntile[2] * c.nspecies; }
+
 size_t cells_args_bytes() { return sizeof(CellsArgs); }
 
 int cells_batch_key(const Ctx &c) { return c.d.shape_order * 4 + c.d.pusher * 2 + (c.any_wall() ? 1 : 0); }
 
-// The tiles of n contexts with one cells_batch_key in one persistent launch of
+// The tiles and species of n contexts with one cells_batch_key in one persistent launch of
 // nsm CTAs on st.  host_args / host_items: pinned host memory of at least
-// n * cells_args_bytes() and (sum of tiles) * 8 bytes, copied to the device
+// n * cells_args_bytes() and (sum of cells_items) * 8 bytes, copied to the device
 // scratch on st (the caller keeps them unchanged until the copy has run).
 cudaError_t launch_particles_cells_batch(Ctx *const *ctxs, int n, cudaStream_t st, CellsBatchScratch &scr,
                                          void *host_args, void *host_items, int nsm) {
@@ -1066,8 +1069,8 @@ cudaError_t launch_particles_cells_batch(Ctx *const *ctxs, int n, cudaStream_t s
     }
     for (int a = 0; a < m; ++a) {
         const Ctx &c = *ctxs[order[a]];
-        const int tiles = c.ntile[0] * c.ntile[1] * c.ntile[2];
-        for (int t = 0; t < tiles; ++t) items[ntot++] = make_int2(a, t);
+        const int n_items = c.ntile[0] * c.ntile[1] * c.ntile[2] * A[a].ns;
+        for (int t = 0; t < n_items; ++t) items[ntot++] = make_int2(a, t);
     }
     if (m == 0) return cudaSuccess;
     const size_t abytes = sizeof(CellsArgs) * (size_t)m, ibytes = sizeof(int2) * (size_t)ntot;

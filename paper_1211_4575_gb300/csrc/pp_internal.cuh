@@ -661,6 +661,7 @@ struct CellsBatchScratch {
     int *next = nullptr;    // work counter
     size_t args_cap = 0, items_cap = 0;
 };
+int64_t cells_items(const Ctx &c);
 int cells_batch_key(const Ctx &c);   // contexts with equal keys can share a launch
 cudaError_t launch_particles_cells_batch(Ctx *const *ctxs, int n, cudaStream_t st, CellsBatchScratch &scr,
                                          void *host_args, void *host_items, int nsm);
