@@ -545,7 +545,7 @@ __device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int item, f
     uint16_t *s_queue = s_piece + kCC + 2;            // crossing particles, in chunk order
     uint16_t *s_xpiece = s_queue + kCC;               // crossing pieces by bucket: first entry | (length - 1) << 12
     int *misc = (int *)(s_grp + kCC);   // [0]: queue length; [2]: pieces;
-                                               // [4..9]: fixed point: cell box of the chunk; [10..12]: sum |dxi|
+                                               // [10..12]: fixed point: sum |dxi|
     int *cnt = misc + 16;                 // starts per (round, warp); four tables
     int *qcnt = cnt + kCPer * kCW;        // crossing particles per (round, warp)
     int *xtot = cnt + 4 * kCPer * kCW;    // crossing pieces per bucket
@@ -597,7 +597,7 @@ __device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int item, f
             const int cn = min(kCC, te - cb);
 #if PP_CELLS_FIXED
             float sum[3] = {0.0f, 0.0f, 0.0f};
-            int blo[3] = {kT, kT, kT}, bhi[3] = {-1, -1, -1};
+            int zlo = kT, zhi = -1;   // cell planes of the chunk's slabs
 #endif
             // ---- phase 1: gather, push, move; write back; stage the deposit
             // the particle of the next round is fetched (through the pending
@@ -624,6 +624,10 @@ __device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int item, f
                     }
                 const int qa = max(cb, s0) - cb, qe = min(cb + cn, s1) - cb;
                 if (qa >= qe) continue;
+#if PP_CELLS_FIXED
+                zlo = min(zlo, slab * kPZ);
+                zhi = slab * kPZ + kPZ - 1;
+#endif
                 fetch(qa + threadIdx.x, qe);
                 __syncthreads();   // the last slab's gathers, or the last chunk's pieces, are done
                 for (int t = threadIdx.x; t < 6 * (kPZ + 4) * kWG; t += kCT) {   // window rows to pairs
@@ -688,8 +692,6 @@ __device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int item, f
                     }
 #if PP_CELLS_FIXED
                     sum[0] += fabsf(dx[0]); sum[1] += fabsf(dx[1]); sum[2] += fabsf(dx[2]);
-                    blo[0] = min(blo[0], rx); blo[1] = min(blo[1], ry); blo[2] = min(blo[2], rz + slab * kPZ);
-                    bhi[0] = max(bhi[0], rx); bhi[1] = max(bhi[1], ry); bhi[2] = max(bhi[2], rz + slab * kPZ);
 #endif
                     // crossing signature: the axis and direction of a support start
                     // that moves on one axis alone, 7 when it moves on several
@@ -722,23 +724,15 @@ __device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int item, f
                 }
             }
 #if PP_CELLS_FIXED
-            if (threadIdx.x < 3) {   // previous chunk's values were last read before the barrier above
-                misc[4 + threadIdx.x] = kT;
-                misc[7 + threadIdx.x] = -1;
-                ((float *)misc)[10 + threadIdx.x] = 0.0f;
-            }
+            // the previous chunk's values were last read before the barrier above
+            if (threadIdx.x < 3) ((float *)misc)[10 + threadIdx.x] = 0.0f;
             __syncthreads();
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 float sd = sum[d];
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) sd += __shfl_xor_sync(0xffffffffu, sd, o);
-                const int l = __reduce_min_sync(0xffffffffu, blo[d]), h = __reduce_max_sync(0xffffffffu, bhi[d]);
-                if (lane == 0) {
-                    atomicAdd((float *)misc + 10 + d, sd);
-                    atomicMin(misc + 4 + d, l);
-                    atomicMax(misc + 7 + d, h);
-                }
+                if (lane == 0) atomicAdd((float *)misc + 10 + d, sd);
             }
 #endif
             __syncthreads();
@@ -882,24 +876,26 @@ __device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int item, f
             }
             __syncthreads();
 #if PP_CELLS_FIXED
-            {   // the window nodes the chunk's cells reach, into the FP32 mesh (and cleared)
-                const int x0 = misc[4], y0 = misc[5], z0 = misc[6];
-                if (misc[7] >= x0) {
-                    const int ex = misc[7] - x0 + kRLo + kRHi + 1, ey = misc[8] - y0 + kRLo + kRHi + 1,
-                              ez = misc[9] - z0 + kRLo + kRHi + 1;
-                    const int vol = ex * ey * ez;
-                    for (int idx = threadIdx.x; idx < 3 * vol; idx += kCT) {
-                        const int comp = idx / vol, r = idx - comp * vol;
-                        const int i = x0 + r % ex, j = y0 + (r / ex) % ey, k = z0 + r / (ex * ey);
+            // the window nodes the chunk's cells reach, into the FP32 mesh (and cleared):
+            // 16 lanes to a row of kW nodes.  Over the exact box of the chunk's cells, by a
+            // flat index, the divisions made this 7 % of the kernel's instructions; the
+            // planes of its slabs, whole, also need no bounds kept per particle (268 M
+            // particle beam 30.08 -> 29.34 ms per step, 192^3 Weibel 19.36 -> 18.91).
+            {
+                const int i = threadIdx.x & 15, rows = (zhi - zlo + kRLo + kRHi + 1) * kW;
+#pragma unroll
+                for (int comp = 0; comp < 3; ++comp)
+                    for (int r = threadIdx.x >> 4; r < rows; r += kCT / 16) {
+                        if (i >= kW) continue;
+                        const int j = r % kW, k = zlo + r / kW;
                         JT *w = Jw + comp * kWVol + wi(i, j, k);
                         const int iv = *w;
                         if (iv == 0) continue;
                         *w = 0;
                         atomicAdd(T.J[comp] + g.at(wx + i, wy + j, wz + k), (float)iv / unit[comp]);
                     }
-                }
-                __syncthreads();
             }
+            __syncthreads();
 #endif
         }
     }
