@@ -583,9 +583,10 @@ __device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int item, f
         }
     }
     for (int idx = threadIdx.x; idx < 3 * kWVol; idx += kCT) Jw[idx] = 0;
-    if (!cta_wait_bounded(bar, phase, kStageWaitNs, T.status)) return false;
-    phase ^= 1;
-    if (misc[3]) return false;
+    // the window has arrived: waited for behind the first particles' loads, two
+    // dependent trips to memory that otherwise start only then (beam 29.37 ->
+    // 28.95 ms per step, 192^3 Weibel 18.95 -> 18.55)
+    bool staged = false;
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     {
@@ -629,6 +630,12 @@ __device__ __forceinline__ bool cells_tile(const CellsArgs &T, const int item, f
                 zhi = slab * kPZ + kPZ - 1;
 #endif
                 fetch(qa + threadIdx.x, qe);
+                if (!staged) {
+                    if (!cta_wait_bounded(bar, phase, kStageWaitNs, T.status)) return false;
+                    phase ^= 1;
+                    if (misc[3]) return false;
+                    staged = true;
+                }
                 __syncthreads();   // the last slab's gathers, or the last chunk's pieces, are done
                 for (int t = threadIdx.x; t < 6 * (kPZ + 4) * kWG; t += kCT) {   // window rows to pairs
                     const int c = t / ((kPZ + 4) * kWG), r = t - c * (kPZ + 4) * kWG;
