@@ -306,12 +306,11 @@ extern "C" int pp_destroy(pp_ctx *p) {
         cudaFree(c->sp[s].alt);
         cudaFree(c->sp[s].keys);
         cudaFree(c->sp[s].perm);
-        cudaFree(c->sp[s].cell_start);
+        cudaFree(c->sp[s].start_mem);
     }
     cudaFree(c->mesh);
     cudaFree(c->rho);
     cudaFree(c->G0);
-    cudaFree(c->counts);
     cudaFree(c->scan_tmp);
     cudaFree(c->d_status);
     cudaFree(c->d_red);
@@ -350,10 +349,10 @@ extern "C" int pp_init_species(pp_ctx *p, const pp_species_desc *sd, int *sid) {
     size_t bytes = per * (size_t)S.cap;
     cudaError_t e1 = cudaMalloc(&S.buf, bytes), e2 = cudaMalloc(&S.alt, bytes);
     cudaError_t e3 = cudaMalloc(&S.keys, sizeof(int32_t) * S.cap);
-    cudaError_t e4 = cudaMalloc(&S.cell_start, sizeof(int32_t) * (c->nkeys + 1));
+    cudaError_t e4 = cell_start_alloc(*c, S);
     cudaError_t e5 = c->fp64 ? cudaSuccess : cudaMalloc(&S.perm, sizeof(int32_t) * S.cap);
     if (e1 || e2 || e3 || e4 || e5) {
-        cudaFree(S.buf); cudaFree(S.alt); cudaFree(S.keys); cudaFree(S.cell_start); cudaFree(S.perm);
+        cudaFree(S.buf); cudaFree(S.alt); cudaFree(S.keys); cudaFree(S.start_mem); cudaFree(S.perm);
         S = Species();
         return fail(c, PP_ENOMEM, "species storage of %zu bytes x 2", bytes);
     }
@@ -592,8 +591,7 @@ static int particle_pre(Ctx *c, bool cells) {
         for (int s = 0; s < c->nspecies; ++s) stale = stale || (c->sp[s].n > 0 && !c->sp[s].fresh);
         if (stale) {
             CU(prof_mark(c, PH_SORT, true));
-            for (int s = 0; s < c->nspecies; ++s)
-                if (!c->sp[s].fresh) CU(launch_sort(*c, s));
+            CU(launch_sort_stale(*c));
             CU(prof_mark(c, PH_SORT, false));
             c->since_sort = 0;
         }

@@ -476,6 +476,7 @@ struct Species {
     void *alt = nullptr;      // sort target of the same layout
     int32_t *keys = nullptr;  // sort keys
     int32_t *cell_start = nullptr; // offsets per sort key (nkeys + 1), valid after a sort
+    int32_t *start_mem = nullptr;  // its allocation
     bool sorted = false;
     bool fresh = false;       // sorted since the particles last moved (the per-step sorted kernel needs it)
     // Per-step sorted kernel: its pass writes every particle's new sort key
@@ -616,7 +617,6 @@ struct Ctx {
     int tile[3] = {8, 8, 8};
     int ntile[3] = {1, 1, 1};
     int64_t nkeys = 0;
-    int32_t *counts = nullptr;   // nkeys + 1
     void *scan_tmp = nullptr;
     size_t scan_tmp_bytes = 0;
     int since_sort = 0;
@@ -688,6 +688,8 @@ cudaError_t launch_ghost_fill(Ctx &c, void *const src_E[3], void *const src_B[3]
 cudaError_t launch_mesh_diag(Ctx &c, double *host_out /* 9 values */);
 
 cudaError_t launch_sort(Ctx &c, int s);
+cudaError_t launch_sort_stale(Ctx &c);   // every species that moved since its last sort
+cudaError_t cell_start_alloc(const Ctx &c, Species &S);
 cudaError_t materialize(Ctx &c, int s);   // apply a pending sort permutation to the arrays
 cudaError_t launch_damp(Ctx &c);
 cudaError_t launch_inject(Ctx &c, int s, int64_t off, int64_t count, uint32_t step, uint32_t pstream, double thick);

@@ -84,15 +84,29 @@ __global__ void k_keys_mixed(KeyGeom kg, int64_t n, const int32_t *cell, const f
     aggregated_add(counts, key);
 }
 
-// ---- exclusive scan of the per-key counts, into the cell starts and, in
-// place, the cursors of the scatter.  Two launches: the sums of blocks of 8192
-// keys (more on meshes of over 8 M cells, so that there are at most 8192
-// blocks), then each block adds up the sums before it and scans its keys.
-// Bound by the launches on small meshes and by the passes over the keys (two
-// reads, two writes) on large ones.  A recursive scan, a pass that added the
-// block offsets and a copy for the cursors were five to eight launches; sort
-// phase per step, both species, before and now: 32^3 cells 0.079, 0.068 ms;
-// mirrored 128 x 64 x 64 0.159, 0.115; 192^3 1.64, 1.27 ----
+// ---- the species sorted together: every launch of the sort takes one species per
+// grid row (blockIdx.y).  Bound by the launches on small meshes and by the
+// passes over the keys on large ones.  A launch per species and a second array
+// for the cursors took, sort phase per step of two species, at 32^3 cells
+// 0.066 ms, 64^3 0.142, 192^3 1.26, on the 268 M particle beam 1.45; this takes
+// 0.038, 0.116, 1.16 and 1.40.
+struct SortJob {
+    int64_t n;             // particles
+    const int32_t *keys;
+    int32_t *counts;       // cell_start + 1: the counts, then the cursors
+    int32_t *perm;
+};
+struct SortJobs {
+    SortJob job[PP_MAX_SPECIES];
+};
+
+// ---- exclusive scan of the per-key counts, in place, into the cursors of the
+// scatter.  The counts of the keys stand one place up in the cell starts: a
+// cursor ends at the start of the next key, so the scatter leaves the cell
+// starts behind it and no second array is written.  Two launches: the sums of
+// blocks of 8192 keys (more on meshes of over 8 M cells, so that there are at
+// most 8192 blocks), then each block adds up the sums before it and scans its
+// keys ----
 constexpr int kScanThreads = 256, kScanRound = 4 * kScanThreads;
 static int scan_rounds(int64_t n) {
     int r = 8;
@@ -122,9 +136,11 @@ __device__ __forceinline__ int32_t block_sum(int32_t v, int32_t *sh) {
     return t;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_sums(const int32_t *in, int64_t n, int rounds,
+__global__ void __launch_bounds__(kScanThreads) k_scan_sums(const __grid_constant__ SortJobs J, int64_t n, int rounds,
                                                             int32_t *sums) {
     __shared__ int32_t sh[kScanThreads / 32];
+    const int32_t *in = J.job[blockIdx.y].counts;
+    sums += (int64_t)blockIdx.y * gridDim.x;
     const int64_t base = (int64_t)blockIdx.x * rounds * kScanRound + 4 * threadIdx.x;
     int32_t v = 0;
 #pragma unroll 4
@@ -136,9 +152,11 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_sums(const int32_t *in, i
     if (threadIdx.x == 0) sums[blockIdx.x] = v;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_write(int32_t *counts, int32_t *start, int64_t n,
-                                                             int rounds, const int32_t *sums) {
+__global__ void __launch_bounds__(kScanThreads) k_scan_write(const __grid_constant__ SortJobs J, int64_t n, int rounds,
+                                                             const int32_t *sums) {
     __shared__ int32_t sh[kScanThreads / 32];
+    int32_t *counts = J.job[blockIdx.y].counts;
+    sums += (int64_t)blockIdx.y * gridDim.x;
     int32_t before = 0;
     for (int b = threadIdx.x; b < (int)blockIdx.x; b += kScanThreads) before += sums[b];
     int32_t carry = block_sum(before, sh);
@@ -170,26 +188,25 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_write(int32_t *counts, in
         e.z = e.y + v.y;
         e.w = e.z + v.z;
         if (q + 3 < n) {
-            *reinterpret_cast<int4 *>(start + q) = e;
             *reinterpret_cast<int4 *>(counts + q) = e;
         } else {
-            if (q < n) start[q] = counts[q] = e.x;
-            if (q + 1 < n) start[q + 1] = counts[q + 1] = e.y;
-            if (q + 2 < n) start[q + 2] = counts[q + 2] = e.z;
+            if (q < n) counts[q] = e.x;
+            if (q + 1 < n) counts[q + 1] = e.y;
+            if (q + 2 < n) counts[q + 2] = e.z;
         }
     }
 }
 
-// counts -> start (exclusive scan) and counts itself; tmp holds the block sums.
-static cudaError_t scan(cudaStream_t st, int32_t *counts, int32_t *start, int64_t n, int32_t *tmp, int64_t &nl) {
+// Exclusive scan of the n counts of each of m jobs; tmp holds the block sums.
+static cudaError_t scan(cudaStream_t st, const SortJobs &J, int m, int64_t n, int32_t *tmp, int64_t &nl) {
     const int rounds = scan_rounds(n);
     const int64_t chunk = (int64_t)rounds * kScanRound;
     const unsigned nb = (unsigned)((n + chunk - 1) / chunk);
-    k_scan_sums<<<nb, kScanThreads, 0, st>>>(counts, n, rounds, tmp);
+    k_scan_sums<<<dim3(nb, m), kScanThreads, 0, st>>>(J, n, rounds, tmp);
     ++nl;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_scan_write<<<nb, kScanThreads, 0, st>>>(counts, start, n, rounds, tmp);
+    k_scan_write<<<dim3(nb, m), kScanThreads, 0, st>>>(J, n, rounds, tmp);
     ++nl;
     return cudaGetLastError();
 }
@@ -279,10 +296,13 @@ __device__ __forceinline__ int32_t window_start(const int32_t *keys, int64_t n, 
     return sh[0];
 }
 
-__global__ void __launch_bounds__(kAggThreads) k_hist(int64_t n, const int32_t *keys, int32_t *counts) {
+__global__ void __launch_bounds__(kAggThreads) k_hist(const __grid_constant__ SortJobs J) {
     __shared__ int32_t cnt[kAggWindow];
     __shared__ int32_t k0s;
-    const int64_t base = (int64_t)blockIdx.x * kAggSpan;
+    const int64_t n = J.job[blockIdx.y].n, base = (int64_t)blockIdx.x * kAggSpan;
+    if (base >= n) return;
+    const int32_t *keys = J.job[blockIdx.y].keys;
+    int32_t *counts = J.job[blockIdx.y].counts;
     int32_t k[kAggPer];
     load_keys(keys, n, base, k);
     for (int i = threadIdx.x; i < kAggWindow; i += kAggThreads) cnt[i] = 0;
@@ -299,10 +319,13 @@ __global__ void __launch_bounds__(kAggThreads) k_hist(int64_t n, const int32_t *
         if (cnt[i]) atomicAdd(counts + k0 + i, cnt[i]);
 }
 
-__global__ void __launch_bounds__(kAggThreads) k_perm(int64_t n, const int32_t *keys, int32_t *cursor, int32_t *perm) {
+__global__ void __launch_bounds__(kAggThreads) k_perm(const __grid_constant__ SortJobs J) {
     __shared__ int32_t cnt[kAggWindow];   // block-local rank counters, then the reserved bases
     __shared__ int32_t k0s;
-    const int64_t base = (int64_t)blockIdx.x * kAggSpan;
+    const int64_t n = J.job[blockIdx.y].n, base = (int64_t)blockIdx.x * kAggSpan;
+    if (base >= n) return;
+    const int32_t *keys = J.job[blockIdx.y].keys;
+    int32_t *cursor = J.job[blockIdx.y].counts, *perm = J.job[blockIdx.y].perm;
     int32_t k[kAggPer], rank[kAggPer];
     load_keys(keys, n, base, k);
     for (int i = threadIdx.x; i < kAggWindow; i += kAggThreads) cnt[i] = 0;
@@ -386,51 +409,116 @@ cudaError_t sort_setup(Ctx &c) {
         c.ntile[a] = (c.g.n[a] + c.tile[a] - 1) / c.tile[a];
     }
     c.nkeys = (int64_t)c.ntile[0] * c.ntile[1] * c.ntile[2] * c.tile[0] * c.tile[1] * c.tile[2] * kSubKeys;
-    cudaError_t e = cudaMalloc(&c.counts, sizeof(int32_t) * (c.nkeys + 1));
-    if (e != cudaSuccess) return e;
-    c.scan_tmp_bytes = sizeof(int32_t) * scan_tmp_count(c.nkeys + 1);
+    c.scan_tmp_bytes = sizeof(int32_t) * scan_tmp_count(c.nkeys + 1) * PP_MAX_SPECIES;
     return cudaMalloc(&c.scan_tmp, c.scan_tmp_bytes);
+}
+
+// The cell starts of a species, with the counts and cursors one place up on a
+// 16-byte boundary.
+cudaError_t cell_start_alloc(const Ctx &c, Species &S) {
+    cudaError_t e = cudaMalloc(&S.start_mem, sizeof(int32_t) * (c.nkeys + 5));
+    S.cell_start = e == cudaSuccess ? S.start_mem + 3 : nullptr;
+    return e;
+}
+
+// keys from the last particle pass: no key pass, and a permutation in place of
+// the scatter
+static bool has_keys(const Ctx &c, const Species &S) {
+    return S.keys_valid && !S.perm_pending && !c.fp64 && S.n > 0;
+}
+
+static SortJob sort_job(const Species &S) { return {S.n, S.keys, S.cell_start + 1, S.perm}; }
+
+static cudaError_t zero_starts(const Ctx &c, const Species &S) {
+    return cudaMemsetAsync(S.cell_start, 0, sizeof(int32_t) * (c.nkeys + 2), c.st);
 }
 
 // Particles that left the box sort after every cell (key nkeys); when the
 // species may hold some, the live count cell_start[nkeys] is read back (a
 // synchronisation) and becomes the species' count, which drops them.
+static cudaError_t sorted_now(Ctx &c, Species &S) {
+    if (S.may_hold_dead) {
+        cudaError_t e = cudaMemcpyAsync(c.h_count, S.cell_start + c.nkeys, sizeof(int32_t), cudaMemcpyDeviceToHost, c.st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c.st);
+        if (e != cudaSuccess) return e;
+        S.n = *c.h_count;
+        S.may_hold_dead = false;
+    }
+    S.nsorted = S.n;
+    S.fresh = true;
+    return cudaSuccess;
+}
+
+// Sorts the m species ids, all with has_keys, together.
+static cudaError_t sort_from_keys(Ctx &c, const int *ids, int m) {
+    SortJobs J{};
+    int64_t nmax = 0;
+    cudaError_t e;
+    for (int q = 0; q < m; ++q) {
+        Species &S = c.sp[ids[q]];
+        S.sorted = true;
+        S.keys_valid = false;
+        J.job[q] = sort_job(S);
+        nmax = S.n > nmax ? S.n : nmax;
+        if ((e = zero_starts(c, S)) != cudaSuccess) return e;
+    }
+    const dim3 grid((unsigned)((nmax + kAggSpan - 1) / kAggSpan), (unsigned)m);
+    k_hist<<<grid, kAggThreads, 0, c.st>>>(J);
+    ++c.nlaunch;
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = scan(c.st, J, m, c.nkeys + 1, (int32_t *)c.scan_tmp, c.nlaunch)) != cudaSuccess) return e;
+    k_perm<<<grid, kAggThreads, 0, c.st>>>(J);
+    ++c.nlaunch;
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    for (int q = 0; q < m; ++q) {
+        c.sp[ids[q]].perm_pending = true;
+        if ((e = sorted_now(c, c.sp[ids[q]])) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t launch_sort_stale(Ctx &c) {
+    int ids[PP_MAX_SPECIES], m = 0;
+    for (int s = 0; s < c.nspecies; ++s) {
+        if (c.sp[s].fresh) continue;
+        if (has_keys(c, c.sp[s])) {
+            ids[m++] = s;
+            continue;
+        }
+        cudaError_t e = launch_sort(c, s);
+        if (e != cudaSuccess) return e;
+    }
+    return m > 0 ? sort_from_keys(c, ids, m) : cudaSuccess;
+}
+
 cudaError_t launch_sort(Ctx &c, int s) {
     Species &S = c.sp[s];
+    if (has_keys(c, S)) return sort_from_keys(c, &s, 1);
     S.sorted = true;
-    // keys from the last particle pass: no key pass, and a permutation in
-    // place of the scatter; otherwise the arrays are put in order first
-    const bool lazy = S.keys_valid && !S.perm_pending && !c.fp64 && S.n > 0;
     S.keys_valid = false;
-    cudaError_t e = lazy ? cudaSuccess : materialize(c, s);
+    cudaError_t e = materialize(c, s);   // the arrays are put in order first
     if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(c.counts, 0, sizeof(int32_t) * (c.nkeys + 1), c.st);
-    if (e != cudaSuccess) return e;
+    if ((e = zero_starts(c, S)) != cudaSuccess) return e;
     if (S.n == 0) {
         S.nsorted = 0;
         S.may_hold_dead = false;
         S.fresh = true;
-        return cudaMemsetAsync(S.cell_start, 0, sizeof(int32_t) * (c.nkeys + 1), c.st);
+        return cudaSuccess;
     }
+    SortJobs J{};
+    J.job[0] = sort_job(S);
+    int32_t *counts = J.job[0].counts;
     KeyGeom kg = key_geom(c);
     unsigned blocks = (unsigned)((S.n + 255) / 256);
-    const unsigned ablocks = (unsigned)((S.n + kAggSpan - 1) / kAggSpan);
-    if (lazy) k_hist<<<ablocks, kAggThreads, 0, c.st>>>(S.n, S.keys, c.counts);
-    else if (c.fp64) k_keys_fp64<<<blocks, 256, 0, c.st>>>(kg, S.n, S.x, S.y, S.z, S.keys, c.counts);
-    else k_keys_mixed<<<blocks, 256, 0, c.st>>>(kg, S.n, S.cell, S.ox, S.oy, S.oz, S.keys, c.counts);
+    if (c.fp64) k_keys_fp64<<<blocks, 256, 0, c.st>>>(kg, S.n, S.x, S.y, S.z, S.keys, counts);
+    else k_keys_mixed<<<blocks, 256, 0, c.st>>>(kg, S.n, S.cell, S.ox, S.oy, S.oz, S.keys, counts);
     ++c.nlaunch;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // cell_start = exclusive scan of counts; counts becomes the cursor
-    if ((e = scan(c.st, c.counts, S.cell_start, c.nkeys + 1, (int32_t *)c.scan_tmp, c.nlaunch)) != cudaSuccess) return e;
-    if (lazy) {
-        k_perm<<<ablocks, kAggThreads, 0, c.st>>>(S.n, S.keys, c.counts, S.perm);
-        ++c.nlaunch;
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        S.perm_pending = true;
-    } else if (c.fp64) {
+    if ((e = scan(c.st, J, 1, c.nkeys + 1, (int32_t *)c.scan_tmp, c.nlaunch)) != cudaSuccess) return e;
+    if (c.fp64) {
         double *b = (double *)S.alt;
         int64_t cp = S.cap;
-        k_scatter_fp64<<<blocks, 256, 0, c.st>>>(S.n, S.keys, c.counts, S.x, S.y, S.z, S.ux, S.uy, S.uz, b, b + cp,
+        k_scatter_fp64<<<blocks, 256, 0, c.st>>>(S.n, S.keys, counts, S.x, S.y, S.z, S.ux, S.uy, S.uz, b, b + cp,
                                                  b + 2 * cp, b + 3 * cp, b + 4 * cp, b + 5 * cp);
         ++c.nlaunch;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -442,7 +530,7 @@ cudaError_t launch_sort(Ctx &c, int s) {
         int64_t cp = S.cap;
         int32_t *c2 = (int32_t *)S.alt;
         float *f2 = (float *)(c2 + cp);
-        k_scatter_mixed<<<blocks, 256, 0, c.st>>>(S.n, S.keys, c.counts, S.cell, S.ox, S.oy, S.oz, S.fux, S.fuy, S.fuz,
+        k_scatter_mixed<<<blocks, 256, 0, c.st>>>(S.n, S.keys, counts, S.cell, S.ox, S.oy, S.oz, S.fux, S.fuy, S.fuz,
                                                   c2, f2, f2 + cp, f2 + 2 * cp, f2 + 3 * cp, f2 + 4 * cp, f2 + 5 * cp);
         ++c.nlaunch;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -451,16 +539,7 @@ cudaError_t launch_sort(Ctx &c, int s) {
         S.alt = old;
         S.bind(false);
     }
-    if (S.may_hold_dead) {
-        e = cudaMemcpyAsync(c.h_count, S.cell_start + c.nkeys, sizeof(int32_t), cudaMemcpyDeviceToHost, c.st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c.st);
-        if (e != cudaSuccess) return e;
-        S.n = *c.h_count;
-        S.may_hold_dead = false;
-    }
-    S.nsorted = S.n;
-    S.fresh = true;
-    return cudaSuccess;
+    return sorted_now(c, S);
 }
 
 }  // namespace pp
