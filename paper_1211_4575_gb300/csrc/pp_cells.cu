@@ -46,10 +46,11 @@
 // FP32 mesh (one global atomic per nonzero node).  A piece's sum is FP32 in
 // registers and is rounded to the unit once.
 //
-// Bound by issue and by the shared-memory pipe behind it: 67 warp-instructions
-// a particle at 50 % of the issue slots (64^3 thermal PCS, 16.8 M particles:
-// 2.25 ms; 95 and 2.62 ms with scalar gathers and sums and the spline weights of
-// each position apart).  On the 268 M particle beam 30.0 ms against 34.2.
+// Bound by issue and by the shared-memory pipe behind it: on the cold beam 67
+// warp-instructions a particle at 50 % of the issue slots, 62 % of the shared
+// pipe.  64^3 thermal PCS, 16.8 M particles, 1.92 ms a step (2.62 with scalar
+// gathers and sums, the spline weights of each position apart and a CTA per
+// tile); 268 M particle beam 28.95 ms against 34.2.
 #include "pp_sorted.cuh"
 #include "pp_tma.cuh"
 
@@ -528,7 +529,10 @@ __device__ __forceinline__ void scan_counts(int *c, int *total, int lane) {
 // species (item: tile times species, plus the species), its current added into
 // the run's mesh.  Called by every thread of the CTA; smem is the CTA's dynamic
 // shared memory.  The chunks of the species are independent, so a species to a
-// CTA changes no sum but makes twice the blocks of a two-species plasma: SPLIT_FIG
+// CTA changes no sum but makes twice the blocks of a two-species plasma, of half
+// the length: 128 CTAs instead of 64 at 32^3 cells (20 steps 6.52 -> 4.58 ms), a
+// shorter last wave at 64^3 (2.25 -> 1.99 ms a step); where the blocks are many, a
+// second staging of the window costs 0.4 % (268 M particle beam).
 // Returns false when the CTA must stop: a staging wait ran out (here or in
 // another CTA, ST_TIMEOUT).  phase: parity of the CTA's staging mbarrier, which
 // the kernel initialised.  GMAPS: the tensor maps sit in global memory.
