@@ -597,8 +597,7 @@ static int particle_pre(Ctx *c, bool cells) {
         }
     }
     CU(launch_zero_J(*c));
-    if (c->nslow_set) CU(cudaMemsetAsync(c->d_nslow, 0, sizeof(unsigned long long), c->st));
-    c->nslow_set = false;
+    c->nslow_counted = false;
     CU(prof_mark(c, PH_PARTICLE, true));
     return PP_OK;
 }
@@ -634,7 +633,10 @@ static int particle_phase(Ctx *c, int only) {
         else CU(launch_particles_rows(*c));
         if (c->prof) ++c->prof_particle_launches;
     } else if (tiled && only < 0) {
-        c->nslow_set = true;   // the only kernel that counts
+        // the only kernel that counts: the counter is cleared in every such pass (and
+        // so in every captured one); after the others pp_diagnostics reports 0
+        CU(cudaMemsetAsync(c->d_nslow, 0, sizeof(unsigned long long), c->st));
+        c->nslow_counted = true;
         CU(launch_particles_tiled_all(*c));
         if (c->prof) ++c->prof_particle_launches;
     } else {
@@ -846,6 +848,7 @@ static void graph_save_after(const Ctx *c, StepGraph &G) {
     G.since_sort_after = c->since_sort;
     G.last_iters = c->last_iters;
     G.last_kk = c->last_kk;
+    G.nslow_counted = c->nslow_counted;
     G.filtered_after_solve = c->filtered_after_solve;
 }
 
@@ -870,6 +873,7 @@ static void graph_apply_after(Ctx *c, const StepGraph &G) {
     }
     c->last_iters = G.last_iters;
     c->last_kk = G.last_kk;
+    c->nslow_counted = G.nslow_counted;
     c->filtered_after_solve = G.filtered_after_solve;
     c->since_sort = G.since_sort_after;
 }
@@ -1186,7 +1190,7 @@ extern "C" int pp_diagnostics(pp_ctx *p, pp_diag *out) {
     out->status = st;
     double mesh[16], kin[PP_MAX_SPECIES];
     unsigned long long nslow = 0;
-    CU(cudaMemcpyAsync(&nslow, c->d_nslow, sizeof nslow, cudaMemcpyDeviceToHost, c->st));
+    if (c->nslow_counted) CU(cudaMemcpyAsync(&nslow, c->d_nslow, sizeof nslow, cudaMemcpyDeviceToHost, c->st));
     CU(launch_rho(*c, true));
     CU(launch_kinetic(*c, c->d_out + 16));
     CU(launch_mesh_diag(*c, mesh));

@@ -525,6 +525,7 @@ struct StepGraph {
     int last_iters = 0;
     double last_kk = 0;
     bool filtered_after_solve = false;
+    bool nslow_counted = false;
 };
 constexpr int kGraphSlots = 8;
 constexpr int kMaxTaps = 64;   // taps of the high-order current's line operator inverse, per axis
@@ -624,7 +625,7 @@ struct Ctx {
     int *d_status = nullptr;
     int *h_status = nullptr;     // pinned mirror
     unsigned long long *d_nslow = nullptr;
-    bool nslow_set = false;      // the last pass counted into it
+    bool nslow_counted = false;  // the last pass counted into it
     unsigned *d_slow_count = nullptr;   // per species, particles left to the global-mesh kernel
     // reductions
     double *d_red = nullptr;     // partials
