@@ -234,7 +234,7 @@ int pp_set_integrator(pp_ctx *ctx, int order);
  * the first time the context is in that state, and replays the capture
  * afterwards.  A state is whether the step sorts, which of the two current
  * buffers holds J, and which of its two buffers holds each species; at most
- * 8 captures are kept, the oldest replaced first.  Results equal those of
+ * 16 captures are kept, the oldest replaced first.  Results equal those of
  * the eager path.  Every call that changes what a step launches (species,
  * particle loads, cooling, integrator, tuning) drops the captures.  Graphs
  * are not used while profiling is enabled.  Needs a context stream other

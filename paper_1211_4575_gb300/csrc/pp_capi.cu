@@ -845,7 +845,6 @@ static void graph_save_after(const Ctx *c, StepGraph &G) {
         G.pending_after[s] = c->sp[s].perm_pending;
         G.keys_valid_after[s] = c->sp[s].keys_valid;
     }
-    G.since_sort_after = c->since_sort;
     G.last_iters = c->last_iters;
     G.last_kk = c->last_kk;
     G.nslow_counted = c->nslow_counted;
@@ -875,7 +874,7 @@ static void graph_apply_after(Ctx *c, const StepGraph &G) {
     c->last_kk = G.last_kk;
     c->nslow_counted = G.nslow_counted;
     c->filtered_after_solve = G.filtered_after_solve;
-    c->since_sort = G.since_sort_after;
+    if (G.sorted_in_step) c->since_sort = 0;   // else the steps since the last sort go on counting
 }
 
 // One step through the graph cache: replay the capture that starts from the
@@ -924,6 +923,7 @@ static int step_graph(Ctx *c, bool sort, bool filter) {
     }
     int since0 = c->since_sort;
     int64_t nl0 = c->nlaunch;
+    c->since_sort = -1;   // a sort in the step sets it to 0
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamBeginCapture(c->st, cudaStreamCaptureModeRelaxed);
     int r = e == cudaSuccess ? step_body(c, sort, filter) : PP_ECUDA;
@@ -949,6 +949,8 @@ static int step_graph(Ctx *c, bool sort, bool filter) {
     }
     G.exec = exec;
     G.launches = (int)(c->nlaunch - nl0);
+    G.sorted_in_step = c->since_sort == 0;
+    if (!G.sorted_in_step) c->since_sort = since0;
     graph_save_after(c, G);
     G.valid = true;
     ++c->graph_captures;

@@ -521,13 +521,15 @@ struct StepGraph {
     void *buf_after[PP_MAX_SPECIES] = {}, *alt_after[PP_MAX_SPECIES] = {};
     bool sorted_after[PP_MAX_SPECIES] = {}, fresh_after[PP_MAX_SPECIES] = {};
     bool pending_after[PP_MAX_SPECIES] = {}, keys_valid_after[PP_MAX_SPECIES] = {};
-    int since_sort_after = 0;
+    bool sorted_in_step = false;   // the step sorted: since_sort starts over
     int last_iters = 0;
     double last_kk = 0;
     bool filtered_after_solve = false;
     bool nslow_counted = false;
 };
-constexpr int kGraphSlots = 8;
+// The states a run steps through: J / J' (B alternates with it), the particle
+// buffer, a sort or none, a filter pass or none.
+constexpr int kGraphSlots = 16;
 constexpr int kMaxTaps = 64;   // taps of the high-order current's line operator inverse, per axis
 
 enum Phase { PH_PARTICLE = 0, PH_CURRENT = 1, PH_FIELD = 2, PH_SORT = 3, PH_N = 4 };

@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 N = (16, 16, 16)
 
 
-def _counts(pp, graphs, steps, sort_interval, current, solver):
+def _counts(pp, graphs, steps, sort_interval, current, solver, filter_interval=0):
     import torch
     L = pp_synth.random_particles(N, (0.5, 0.5, 0.5), 0.2, 4000, seed=77, u_scale=3.0, w=1e-12)
     stream = torch.cuda.Stream()
@@ -26,6 +26,8 @@ def _counts(pp, graphs, steps, sort_interval, current, solver):
         sim.load_particles(sid, s["x"], s["y"], s["z"], s["ux"], s["uy"], s["uz"])
     sim.set_current_deposit(current)
     sim.set_field_solver(solver)
+    if filter_interval:
+        sim.set_divergence_filter(1, filter_interval)
     sim.set_graphs(graphs)
     out = []
     for _ in range(steps):
@@ -69,3 +71,30 @@ def test_slow_count_is_zero_after_passes_of_another_kernel():
         for _ in range(4):
             sim.step(1)
             assert sim.diagnostics()["n_slow"] == 0
+
+
+def test_periodic_sorts_go_on_in_replayed_steps():
+    """A sort every 4 steps for 24 steps: a replay of a step without a sort
+    does not set the count of steps since the last sort back, so the sorts keep
+    their interval and the particles outside their tiles stay as few as in the
+    eager run."""
+    import paper_1211_4575_gb300 as pp
+    cur, sol = pp.PP_CURRENT_DIRECT, pp.PP_FIELD_EXPLICIT
+    eager, _ = _counts(pp, False, 24, 4, cur, sol)
+    graph, (cap, rep) = _counts(pp, True, 24, 4, cur, sol)
+    unsorted, _ = _counts(pp, False, 24, 0, cur, sol)
+    assert rep >= 8, (cap, rep)
+    assert unsorted[-1] > 10 * max(1, eager[-1])   # the counts tell the sorts apart
+    assert graph == eager
+
+
+def test_captures_of_a_long_cycle_are_kept():
+    """Tiled, a sort every 4 and a filter every 3 steps: the run cycles through
+    12 states (current array, particle buffer, sort, filter), and once all are
+    captured every step is a replay."""
+    import paper_1211_4575_gb300 as pp
+    cur, sol = pp.PP_CURRENT_CONSERVING, pp.PP_FIELD_IMPLICIT
+    eager, _ = _counts(pp, False, 48, 4, cur, sol, filter_interval=3)
+    graph, (cap, rep) = _counts(pp, True, 48, 4, cur, sol, filter_interval=3)
+    assert cap <= 16 and rep >= 32, (cap, rep)
+    assert graph == eager
