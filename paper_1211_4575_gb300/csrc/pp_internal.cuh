@@ -97,12 +97,14 @@ __device__ __forceinline__ int support(R xi, bool half, R (&w)[O + 1]) {
 
 // 1 / sqrt(x), x >= 1.  FP32: one Newton-Raphson step on the hardware estimate
 // (y += y/2 (1 - x y^2), error below one ulp), a quarter of the instructions of
-// a correctly rounded square root and division; infinity gives 0.
+// a correctly rounded square root and division; infinity gives 0.  Only infinity
+// (and NaN) leaves out the step: every finite x takes it.
+constexpr float kFloatMax = 3.402823466e38f;
 __device__ __forceinline__ double inv_sqrt(double x) { return 1.0 / sqrt(x); }
 __device__ __forceinline__ float inv_sqrt(float x) {
     const float y = rsqrtf(x);
     const float r = fmaf(0.5f * y, fmaf(-(x * y), y, 1.0f), y);
-    return x < 3.0e38f ? r : y;
+    return x <= kFloatMax ? r : y;
 }
 
 // sqrt(x) of x > 0 and 1 / x of x >= 1, likewise.
@@ -110,12 +112,14 @@ __device__ __forceinline__ double fast_sqrt(double x) { return sqrt(x); }
 __device__ __forceinline__ float fast_sqrt(float x) {
     const float y = rsqrtf(x), s = x * y;
     const float r = fmaf(0.5f * y, fmaf(-s, s, x), s);
-    return x < 3.0e38f ? r : x;
+    return x <= kFloatMax ? r : x;
 }
 __device__ __forceinline__ double inv(double x) { return 1.0 / x; }
 __device__ __forceinline__ float inv(float x) {
-    const float y = __fdividef(1.0f, x);
-    return x < 1.0e38f ? fmaf(y, fmaf(-x, y, 1.0f), y) : y;
+    // the estimate is 0 for x > 2^126, whose reciprocal is subnormal: scaled by 1/8 there
+    const float s = x > 8.0e37f ? 0.125f : 1.0f, xs = x * s;
+    const float y = __fdividef(1.0f, xs);
+    return (x <= kFloatMax ? fmaf(y, fmaf(-xs, y, 1.0f), y) : y) * s;
 }
 
 // ---------------------------------------------------------------------------
