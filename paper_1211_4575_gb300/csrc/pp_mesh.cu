@@ -683,14 +683,9 @@ __global__ void __launch_bounds__(256) k_cheb(Geom g, const __grid_constant__ Co
 // iterate, the previous one and the right-hand side in shared memory, read the
 // planes above and below from one another's shared memory and meet at the
 // cluster's hardware barrier after each sweep.  Sweeps of their own cost 6.3 us
-// (FP32) to 8.4 us (FP64) each however small the mesh.  Whole field update, in
-// launches and in one cluster: 16^3 FP32 94, 33 us; 32^3 101, 56; 40^3 136, 95;
-// 48 x 40 x 32 132, 89; 48^3 165, 165; FP64 16^3 201, 103; 20^3 209, 279.  Past
-// the line the launches win: they use all SMs, the clusters 48, and FP64 is
-// bound by its rate.
+// (FP32) to 8.4 us (FP64) each however small the mesh; past a line they win all
+// the same: they use all SMs, the clusters 48 (cluster_pays).
 constexpr int kClusterCtas = 16, kClusterThreads = 512, kClusterSweeps = 64;
-template <typename R>
-constexpr int kClusterNodes = sizeof(R) == 4 ? 70000 : 6000;
 
 template <typename R>
 struct Sweeps {
@@ -839,11 +834,42 @@ __global__ void __launch_bounds__(kClusterThreads, 1)
     }
 }
 
+// Whether the cluster is faster than a launch per sweep: both estimated in us
+// from measurements of the whole field update (dt = dx / 2; tolerance 1e-6 in
+// FP32, 1e-12 in FP64).  What counts in the cluster is the heaviest CTA, with p
+// planes: its warps' columns and, for each, the 11 nodes fetched before the
+// march and the planes marched; with W = 1 a column holds half the work.  In
+// FP64 a warp's rate shows from four warps on (below them its latency), and a
+// second pass over the columns costs a full one.  Launches and cluster, us:
+//   FP32 16^3 96, 33; 32^3 102, 58; 32 x 32 x 224 215, 156; 41^3 136, 115;
+//   48^3 167, 122; 64 x 48 x 16 102, 105; 64 x 64 x 16 119, 126; 64 x 64 x 17
+//   115, 165 (8192 nodes in one CTA, 4096 in the others); 52 x 54 x 17 103, 124;
+//   61 x 61 x 17 134, 184; 63 x 47 x 33 137, 164.
+//   FP64 16^3 203, 105; 8 x 8 x 64 211, 281; 9 x 9 x 64 202, 167; 12 x 12 x 48
+//   204, 222; 16 x 20 x 17 203, 226; 17^3 202, 190; 20^3 212, 281;
+//   24 x 24 x 16 212, 199; 28 x 24 x 16 211, 230.
+// Of 148 meshes measured the estimates choose the slower form (by over 3 %) five
+// times, by 4 to 20 %; limits of 70,000 and 6,000 nodes in all chose it 61 times.
+template <typename R, int W>
+static bool cluster_pays(const Geom &g) {
+    const int p = (g.n[2] + kClusterCtas - 1) / kClusterCtas, cols = g.n[0] / W * g.n[1];
+    int warps = (cols + 31) / 32;
+    if (sizeof(R) == 4) {
+        const double launches = 70.0 + 0.65e-3 * (double)g.cells();
+        return 27.0 + warps * (W == 2 ? 1.0 : 0.62) * (1.1 + 0.45 * p) <= (launches > 100.0 ? launches : 100.0);
+    }
+    constexpr int kPass = kClusterThreads / 32;
+    if (warps > kPass) warps = (warps + kPass - 1) / kPass * kPass;
+    if (warps < 4) warps = 4;
+    return 38.0 + p * warps * (W == 2 ? 17.3 : 7.7) <= 201.0;
+}
+
 template <typename R, int W>
 static bool cluster_fits(const Geom &g, int sweeps, size_t &smem) {
     const int pmax = (g.n[2] + kClusterCtas - 1) / kClusterCtas;
     smem = (size_t)3 * pmax * g.n[0] * g.n[1] * sizeof(R);
-    if (g.n[0] < 8 || g.n[1] < 8 || g.n[2] < kClusterCtas || pmax + 10 > 24 || sweeps > kClusterSweeps || g.cells() > kClusterNodes<R> || smem > 224 * 1024)
+    if (g.n[0] < 8 || g.n[1] < 8 || g.n[2] < kClusterCtas || pmax + 10 > 24 || sweeps > kClusterSweeps || smem > 224 * 1024 ||
+        !cluster_pays<R, W>(g))
         return false;
     // once per device and kernel: whether the three clusters can be resident
     static unsigned long long asked = 0, ok = 0;
