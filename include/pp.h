@@ -83,7 +83,9 @@ extern "C" {
                                 multiples of 8; PP_DEPOSIT_AUTO takes it wherever it
                                 applies, and on other meshes of at least 8 cells
                                 per axis a kernel of rows of cells that sorts in
-                                every pass as well and sums the current in FP32     */
+                                every pass as well and sums the current in FP32,
+                                where the particles are many enough to pay for the
+                                sort (else PP_DEPOSIT_GLOBAL's kernel and interval) */
 
 #define PP_FIELD_IMPLICIT 0  /* de-centred implicit update, eq:EllipticB (default)    */
 #define PP_FIELD_EXPLICIT 1  /* explicit FDTD leap-frog (cold-beam comparison)         */

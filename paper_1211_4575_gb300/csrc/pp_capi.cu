@@ -458,6 +458,7 @@ extern "C" int pp_load_particles(pp_ctx *p, int sid, int64_t n, const double *x,
     if (rc != PP_OK) return rc;
     S.n += n;
     CU(launch_sort(*c, sid));
+    if (rows_supported(*c)) CU(count_tiles_held(*c, sid));
     if (!c->slab) c->g0_pending = true;   // a slab rank's rho is a share: no reference
     return PP_OK;
 }
@@ -576,9 +577,10 @@ static bool cells_mode(const Ctx *c) {
 }
 
 // Either kernel that starts from particles sorted in this step: that one, or
-// on meshes its tiles do not divide the row kernel (automatic deposit).
+// on meshes its tiles do not divide the row kernel (automatic deposit, where
+// the load pays for the sort and the windows).
 static bool sorted_mode(const Ctx *c) {
-    return cells_mode(c) || (c->d.deposit_mode == PP_DEPOSIT_AUTO && rows_supported(*c));
+    return cells_mode(c) || (c->d.deposit_mode == PP_DEPOSIT_AUTO && rows_supported(*c) && rows_pay(*c));
 }
 
 // The parts of a particle phase around its kernel launch: before it, the

@@ -481,6 +481,7 @@ struct Species {
     int32_t *keys = nullptr;  // sort keys
     int32_t *cell_start = nullptr; // offsets per sort key (nkeys + 1), valid after a sort
     int32_t *start_mem = nullptr;  // its allocation
+    int64_t tiles_held = 0;   // sort tiles that held particles at the last load (rows_pay)
     bool sorted = false;
     bool fresh = false;       // sorted since the particles last moved (the per-step sorted kernel needs it)
     // Per-step sorted kernel: its pass writes every particle's new sort key
@@ -660,6 +661,7 @@ cudaError_t launch_particles_cells(Ctx &c);
 bool cells_supported(const Ctx &c);
 cudaError_t launch_particles_rows(Ctx &c);
 bool rows_supported(const Ctx &c);
+bool rows_pay(const Ctx &c);   // whether the automatic deposit takes it there
 // batched form: one launch over the tiles of many contexts (same shape order,
 // pusher and boundary kind); scratch = device memory the caller owns
 struct CellsBatchScratch {
@@ -697,6 +699,7 @@ cudaError_t launch_mesh_diag(Ctx &c, double *host_out /* 9 values */);
 cudaError_t launch_sort(Ctx &c, int s);
 cudaError_t launch_sort_stale(Ctx &c);   // every species that moved since its last sort
 cudaError_t cell_start_alloc(const Ctx &c, Species &S);
+cudaError_t count_tiles_held(Ctx &c, int s);   // of a species just sorted; synchronises
 cudaError_t materialize(Ctx &c, int s);   // apply a pending sort permutation to the arrays
 cudaError_t launch_damp(Ctx &c);
 cudaError_t launch_inject(Ctx &c, int s, int64_t off, int64_t count, uint32_t step, uint32_t pstream, double thick);

@@ -652,6 +652,41 @@ bool rows_supported(const Ctx &c) {
     return !divided;
 }
 
+// Whether the row kernel and its sort take less time than the global-mesh kernel
+// with a sort every 20 steps, the other route of the automatic deposit on such
+// meshes.  The sort and the empty blocks cost by the mesh, the windows and rows
+// by the tiles that hold particles, the global kernel by the particle: about
+// 0.1, 0.3 and 0.9 ns (CIC, TSC, PCS), less where a launch is too small to fill
+// the GPU.  So the line is a count of particles, n0 + a tiles of the fullest
+// species + b tiles of all + c tiles of the mesh (in cells).  Particle phase and
+// sort of two thermal species together, row and global kernel, ms a step:
+//   163 x 161 x 157, 4 per cell: CIC 4.38, 1.59; TSC 5.55, 5.80; PCS 6.32, 14.5
+//                    0.1 per cell, PCS: 3.29, 0.49; 1 per cell: 4.75, 3.53
+//   60 x 45 x 37, 16 per cell: CIC 0.237, 0.166; TSC 0.318, 0.666; PCS 0.370, 1.76
+//                 1 per cell, PCS: 0.190, 0.136; 2 per cell: 0.197, 0.198
+//   20^3, 4 per cell: CIC 0.082, 0.022; TSC 0.090, 0.040; PCS 0.094, 0.078
+// A hot plasma (u = 2) tips the balance at half the load of a thermal one; the
+// line lies between the two.  Above `most` particles per cell the row kernel is
+// taken all the same: the global kernel's error grows with the particles that
+// add to a node one by one (J of counter-streaming electrons and ions against
+// FP64, row and global: 32 per cell PCS 7e-7, 2.3e-6, TSC 6e-7, 1.3e-6, CIC
+// 6e-7, 7e-7; 8 per cell PCS 7e-7, 9e-7).
+bool rows_pay(const Ctx &c) {
+    static constexpr double n0[4] = {0, 250e3, 80e3, 30e3}, a[4] = {0, 3.0, 0.9, 0.45}, b[4] = {0, 2.7, 0.65, 0.3},
+                            m[4] = {0, 1.0, 0.3, 0.1}, most[4] = {0, 48, 8, 8};
+    const int o = c.d.shape_order;
+    double n = 0.0, fullest = 0.0, held = 0.0;
+    for (int s = 0; s < c.nspecies; ++s) {
+        const double h = (double)c.sp[s].tiles_held * kSortTileCells;
+        n += (double)c.sp[s].n;
+        held += h;
+        fullest = h > fullest ? h : fullest;
+    }
+    const double mesh = (double)c.ntile[0] * c.ntile[1] * c.ntile[2] * kSortTileCells;
+    const double filled = fullest < (double)c.g.cells() ? fullest : (double)c.g.cells();
+    return n >= n0[o] + a[o] * fullest + b[o] * held + m[o] * mesh || n >= most[o] * filled;
+}
+
 // All species in one launch; every species with particles must have been
 // sorted since its particles last moved (Species::fresh).
 cudaError_t launch_particles_rows(Ctx &c) {

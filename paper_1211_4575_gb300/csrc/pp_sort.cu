@@ -477,6 +477,30 @@ static cudaError_t sort_from_keys(Ctx &c, const int *ids, int m) {
     return cudaSuccess;
 }
 
+__global__ void k_tiles_held(int ntiles, int64_t tile_keys, const int32_t *cell_start, int32_t *held) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool any = t < ntiles && cell_start[(t + 1) * tile_keys] > cell_start[t * tile_keys];
+    const unsigned m = __ballot_sync(0xffffffffu, any);
+    if ((threadIdx.x & 31) == 0 && m) atomicAdd(held, __popc(m));
+}
+
+cudaError_t count_tiles_held(Ctx &c, int s) {
+    Species &S = c.sp[s];
+    S.tiles_held = 0;
+    if (S.n == 0) return cudaSuccess;
+    const int ntiles = c.ntile[0] * c.ntile[1] * c.ntile[2];
+    int32_t *held = (int32_t *)c.scan_tmp;   // free between sorts
+    cudaError_t e = cudaMemsetAsync(held, 0, sizeof(int32_t), c.st);
+    if (e != cudaSuccess) return e;
+    k_tiles_held<<<(ntiles + 255) / 256, 256, 0, c.st>>>(ntiles, c.nkeys / ntiles, S.cell_start, held);
+    ++c.nlaunch;
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = cudaMemcpyAsync(c.h_count, held, sizeof(int32_t), cudaMemcpyDeviceToHost, c.st)) != cudaSuccess) return e;
+    if ((e = cudaStreamSynchronize(c.st)) != cudaSuccess) return e;
+    S.tiles_held = *c.h_count;
+    return cudaSuccess;
+}
+
 cudaError_t launch_sort_stale(Ctx &c) {
     int ids[PP_MAX_SPECIES], m = 0;
     for (int s = 0; s < c.nspecies; ++s) {
