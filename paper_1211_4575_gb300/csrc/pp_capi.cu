@@ -605,8 +605,13 @@ static int particle_pre(Ctx *c, bool cells) {
 }
 
 static int particle_post(Ctx *c, int only) {
-    for (int s = 0; s < c->nspecies; ++s)
-        if (only < 0 || s == only) c->sp[s].fresh = false;   // the particles moved
+    for (int s = 0; s < c->nspecies; ++s) {
+        if (only >= 0 && s != only) continue;
+        c->sp[s].fresh = false;   // the particles moved
+        // those that this pass took out of the box stay in the arrays until a sort (the
+        // sort before the pass dropped the earlier ones)
+        if (c->escape_now > 0.0) c->sp[s].may_hold_dead = true;
+    }
     CU(prof_mark(c, PH_PARTICLE, false));
     CU(prof_mark(c, PH_CURRENT, true));
     CU(launch_fold_J(*c));
@@ -787,8 +792,6 @@ static int step_body(Ctx *c, bool sort, bool filter) {
     int r = PP_OK;
     // the open end takes outgoing particles at the end of a full step
     const double esc = (c->wall[0] && c->open.cells > 0) ? c->open.escape : 0.0;
-    if (esc > 0.0)
-        for (int s = 0; s < c->nspecies; ++s) c->sp[s].may_hold_dead = true;
     if (c->order == 4) {
         double a[4], b[4];
         step4_fractions(a, b);
