@@ -972,7 +972,12 @@ extern "C" int pp_step(pp_ctx *p, int nsteps) {
         bool sort = c->d.sort_interval > 0 && c->since_sort >= c->d.sort_interval;
         bool filter = c->filter_passes > 0 && (c->step + 1) % c->filter_interval == 0;
         const bool dyn = boundary_dynamic(c);
-        int r = (c->use_graphs && !c->prof && c->st && !dyn) ? step_graph(c, sort, filter) : step_body(c, sort, filter);
+        const bool graph = c->use_graphs && !c->prof && c->st && !dyn;
+        int r = PP_OK;
+        // particles that left before the open end was closed: the sort that drops them
+        // reads a count back, which a capture cannot hold
+        if (graph) r = compact(c);
+        if (r == PP_OK) r = graph ? step_graph(c, sort, filter) : step_body(c, sort, filter);
         if (r) return r;
         ++c->step;
         ++c->since_sort;
