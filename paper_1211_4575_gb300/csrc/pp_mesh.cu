@@ -7,6 +7,8 @@
 // filled (the particle gather reads them), and so do the relaxation iterates:
 // the implicit solver's stencils read those through linear offsets.
 // Other stencils read interior values through periodic wrapping (Nb).
+#include <atomic>
+
 #include "pp_internal.cuh"
 
 namespace pp {
@@ -871,12 +873,13 @@ static bool cluster_fits(const Geom &g, int sweeps, size_t &smem) {
     if (g.n[0] < 8 || g.n[1] < 8 || g.n[2] < kClusterCtas || pmax + 10 > 24 || sweeps > kClusterSweeps || smem > 224 * 1024 ||
         !cluster_pays<R, W>(g))
         return false;
-    // once per device and kernel: whether the three clusters can be resident
-    static unsigned long long asked = 0, ok = 0;
+    // once per device and kernel: whether a cluster can be resident (contexts may
+    // step from several threads: a thread that sees `asked` also sees `ok`)
+    static std::atomic<unsigned long long> asked{0}, ok{0};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
     const unsigned long long bit = 1ull << (dev & 63);
-    if (!(asked & bit)) {
+    if (!(asked.load(std::memory_order_acquire) & bit)) {
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -892,10 +895,10 @@ static bool cluster_fits(const Geom &g, int sweeps, size_t &smem) {
                    cudaFuncSetAttribute(k_cheb_cluster<R, W>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
                    cudaOccupancyMaxActiveClusters(&n, k_cheb_cluster<R, W>, &cfg) == cudaSuccess && n >= 1;
         if (!can) cudaGetLastError();
-        if (can) ok |= bit;
-        asked |= bit;
+        if (can) ok.fetch_or(bit, std::memory_order_relaxed);
+        asked.fetch_or(bit, std::memory_order_release);
     }
-    return (ok & bit) != 0;
+    return (ok.load(std::memory_order_relaxed) & bit) != 0;
 }
 
 // E_new = E + dt (curl^- (alpha B_new + beta B_old) - J), ghosts of E included.
