@@ -47,16 +47,16 @@ BYTES_PER_PARTICLE_STEP = 56   # mixed form: (int32 cell + 3 fp32 offsets + 3 fp
 # are the ones it was taken on (sha256 below); otherwise the line reports
 # traffic, limiter and issue as null.
 PROFILED = {
-    "beam": {"bytes_per_particle": 64.34, "warp_inst_per_particle": 67.2,
+    "beam": {"bytes_per_particle": 64.32, "warp_inst_per_particle": 67.4,
              "limiter": "instruction issue and the shared-memory pipe (49.9 % of issue slots busy; shared pipe "
-                        "61.6 %, FMA 27.7 % of peak; DRAM 7.3 %)"},
-    "thermal": {"bytes_per_particle": 64.06, "warp_inst_per_particle": 64.3,
+                        "61.5 %, FMA 27.7 % of peak; DRAM 7.2 %)"},
+    "thermal": {"bytes_per_particle": 64.10, "warp_inst_per_particle": 64.4,
                 "limiter": "instruction issue and the shared-memory pipe (47.2 % of issue slots busy; shared pipe "
-                           "60.6 %, FMA 25.2 % of peak; DRAM 7.1 %)"},
+                           "60.4 %, FMA 25.1 % of peak; DRAM 7.1 %)"},
 }
 PROFILED_SOURCES = {
     "paper_1211_4575_gb300/csrc/pp_cells.cu": "1d43f71e50f9c1a38d43138239a8b483d4bc06d8e91e6a406eaef953d24676c1",
-    "paper_1211_4575_gb300/csrc/pp_internal.cuh": "a6087a7d920e4c12d27695749257e31afaae8f28517dc73a8eabe3895cf93fcf",
+    "paper_1211_4575_gb300/csrc/pp_internal.cuh": "914b5b7b8723fcf95af1c2fd24c29af9f063d6ada985e64a5d32c7fbde552188",
     "paper_1211_4575_gb300/csrc/pp_particle_common.cuh": "6805ab903ef2be60e620b6059392d7afd2da3fd0f9a098f8dbf04858b8b05717",
     "paper_1211_4575_gb300/csrc/pp_sorted.cuh": "31194ab332621153ecaf979aadb4c134c02d92645d9a384c90dc220327e0c945",
     "paper_1211_4575_gb300/csrc/pp_tma.cuh": "e0ac1f2401ee66da9f6509e7830a148f7aadb33c4eab9f1a62bf6f1a7995817c",

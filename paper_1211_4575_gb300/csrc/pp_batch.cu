@@ -69,7 +69,8 @@ static void release(pp_batch *b, pp_batch::Slot &S) {
 // between walls) with the given rounded species capacities: 21 padded mesh
 // arrays, the compact rho and Gauss reference, and per species two particle
 // buffers, the sort keys (and, in the mixed form, the permutation) and the
-// per-key offsets, plus the sort's counters.
+// per-key offsets, plus four bytes a key for the sort: an upper bound, since the
+// sort counts in the offsets and holds only its block sums besides.
 static int64_t context_bytes(const int n[3], bool fp64, int ns, const int64_t *cap) {
     int64_t padded = 1, cells = 1, nkeys = kSubKeys;
     for (int a = 0; a < 3; ++a) {

@@ -821,7 +821,8 @@ static int step_body(Ctx *c, bool sort, bool filter) {
 static bool graph_matches(const Ctx *c, const StepGraph &G, bool sort, bool filter) {
     if (!G.valid || G.sort != sort || G.filter != filter || G.J0 != c->J[0] || G.B0 != c->B[0]) return false;
     // freshness, a pending permutation and valid keys change what a step
-    // launches only for the per-step sorted kernels (elsewhere they stay false)
+    // launches only for the per-step sorted kernels (elsewhere nothing reads them
+    // before the pass clears them, though a filter's sort sets freshness)
     const bool cells = sorted_mode(c);
     for (int s = 0; s < c->nspecies; ++s) {
         if (G.buf[s] != c->sp[s].buf || G.sorted[s] != c->sp[s].sorted) return false;

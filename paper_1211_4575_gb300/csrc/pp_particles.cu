@@ -62,12 +62,15 @@ struct StepArgs {
 // support moves, but one of them makes its whole warp run it.  The block
 // therefore compacts its particles through shared memory: those that cross no
 // support boundary first, with the form on O + 1 nodes, then the others: 1406
-// FP64 instructions per warp instead of 1680 (PCS, Vay, thermal).  Splitting the
-// two passes also lets the registers fit two blocks per SM.  800 k particles on
-// 45 x 30 x 37 cells: 2.71 -> 2.33 ms per step (one block per SM 2.61; 128
-// threads 2.54 at three blocks, 2.57 at four; 64 threads 2.54; 192 threads 2.28,
-// but 0.203 instead of 0.155 ms for the 65 k particles of 16^3 cells, two rounds
-// of blocks there).
+// FP64 instructions per warp instead of 1680 (PCS, Vay, thermal).  Two blocks per
+// SM are the faster even though their 128 registers do not hold a PCS particle
+// (992 bytes of stack; 2.4 KB of spill stores and 3.5 KB of loads a thread; TSC
+// 308 and 416 bytes, CIC none).  800 k particles on 45 x 30 x 37 cells: 2.71 ->
+// 2.33 ms per step (one block per SM 2.61; 128 threads 2.54 at three blocks, 2.57
+// at four; 64 threads 2.54; 192 threads 2.28, but 0.203 instead of 0.155 ms for
+// the 65 k particles of 16^3 cells, two rounds of blocks there).  A plasma whose
+// particles nearly all cross gains nothing (32^3 x 16 at u_x = 10, a step of 0.9
+// cells: 1.82 -> 1.87 ms).
 constexpr int kFp64Threads = 256;
 template <int O, int PUSH>
 __global__ void __launch_bounds__(kFp64Threads, 2) k_particles_fp64(StepArgs<double> a, Fp64Particles p) {

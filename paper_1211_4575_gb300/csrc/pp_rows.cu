@@ -3,10 +3,10 @@
 // (Sec. III: the paper sorts the particle array by cell position in every
 // step, between the current deposit and the field update).
 //
-// Such meshes took one thread per particle on the global mesh, with an L2
-// reduction per site (144 of them for a PCS particle): 3.89 ms per step for
-// 3.2 M particles on 60 x 45 x 37 cells, against 0.54 ms here (and 0.09 ms for
-// the sort).
+// The other kernel of such meshes takes one thread per particle on the global
+// mesh, with an L2 reduction per site (144 of them for a PCS particle): 3.89 ms
+// per step for 3.2 M particles on 60 x 45 x 37 cells, against 0.54 ms here (and
+// 0.06 ms for the sort).  Few particles stay with it (rows_pay).
 //
 // One CTA of 16 warps per block of 8 x 8 x tz cells (tz = 4, 2 or 1: a slab of
 // an 8^3 tile of the sort, whose particles are contiguous; the last tiles are
@@ -36,7 +36,8 @@
 // as packed pairs.
 //
 // Bound by issue: 82 warp-instructions a particle at 60 % of the issue slots
-// (64^3 thermal PCS).  Emitting nodes four at a time through a shared ring, as
+// (64^3 thermal PCS; 128 registers, of which PCS spills some 30 bytes a thread
+// and TSC 116).  Emitting nodes four at a time through a shared ring, as
 // vector reductions, was slower: more code than the instruction cache holds.
 #include "pp_sorted.cuh"
 
@@ -637,11 +638,12 @@ __global__ void __launch_bounds__(kCT, 1) k_particles_rows(const __grid_constant
 }  // namespace
 
 // Mixed form, charge-conserving current, every size at least one 8-cell tile,
-// and some size no multiple of 8: the automatic deposit takes this kernel.
-// Meshes that the tiles divide keep the tile kernel of pp_cells.cu, and with it
-// the rounding their runs have had: its fixed-point sums leave up to 2e-5 of a
-// weak net current (counter-streaming beams), twenty times this kernel's error,
-// at the same speed (64^3 thermal PCS: 1.96 ms here).
+// and some size no multiple of 8.  On meshes that the tiles divide the tile
+// kernel of pp_cells.cu serves, which the batched runs share: as fast at 64
+// thermal PCS particles a cell (64^3: 1.93 ms, this one 1.96) though less exact
+// where a net current is weak (its fixed-point sums leave up to 2e-5 of it in
+// counter-streaming beams, this kernel 1e-6).  The two have not been compared at
+// other loads.
 bool rows_supported(const Ctx &c) {
     if (c.fp64 || c.current_mode != PP_CURRENT_CONSERVING || c.g.G < kWG - kT - kRLo) return false;
     bool divided = true;
